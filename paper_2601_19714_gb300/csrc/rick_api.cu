@@ -924,8 +924,10 @@ Occupancy plan_occupancy(const rick_plan* P) {
 }
 
 // Pass 1 of the own transform (inverse DFT down every column), in place.
+// own: grids is the plan's own memory: only the image's rows of the result are
+// stored (nothing reads the other rows of a padded mesh).
 rick_status columns_impl(rick_plan* P, float* grids, int c0, int c1, int k0, int k1, int32_t flags,
-                         cudaStream_t st) {
+                         cudaStream_t st, bool own = false) {
     const rick_config& c = P->cfg;
     if (!P->own_fft) {
         set_err("the column pass needs the library's own transform (RICK_FFT_OWN, a mesh of 256 to 16384)");
@@ -942,9 +944,11 @@ rick_status columns_impl(rick_plan* P, float* grids, int c0, int c1, int k0, int
         occ = plan_occupancy(P);
     }
     int launches = 0;
+    const int off = own ? (P->Ng - c.N) / 2 : 0;
     rick_status s = check_launch(launch_fft_columns(reinterpret_cast<float2*>(grids),
                                                     (int64_t)(c1 - c0) * (k1 - k0), P->Ng, true,
-                                                    P->d_twid, occ, st, &launches, fourstep_layout(P)),
+                                                    P->d_twid, occ, st, &launches, fourstep_layout(P),
+                                                    off, P->Ng - off),
                                  "FFT column kernel");
     P->launches += launches;
     return s;
@@ -985,7 +989,7 @@ rick_status rows_phase_impl(rick_plan* P, const float* grids, int c0, int c1, in
 // [c0, c1): with the own transform, the column pass and the fused row pass.
 rick_status fft_phase_impl(rick_plan* P, float* grids, int c0, int c1, int k0, int k1,
                            const double* weight_sum, float* image_real, float* image_complex,
-                           cudaStream_t st, int32_t flags = 0) {
+                           cudaStream_t st, int32_t flags = 0, bool own = false) {
     const rick_config& c = P->cfg;
     if (!P->own_fft) {
         RK_ARG(0 <= c0 && c0 < c1 && c1 <= c.n_channels, "channel range");
@@ -995,7 +999,7 @@ rick_status fft_phase_impl(rick_plan* P, float* grids, int c0, int c1, int k0, i
     }
     RK_ARG(0 <= c0 && c0 < c1 && c1 <= c.n_channels, "channel range");
     RK_ARG(0 <= k0 && k0 < k1 && k1 <= P->planes, "plane range");
-    RK_TRY(columns_impl(P, grids, c0, c1, k0, k1, flags, st));
+    RK_TRY(columns_impl(P, grids, c0, c1, k0, k1, flags, st, own));
     // the occupancy computed by the column pass serves the row pass too
     return rows_phase_impl(P, grids, c0, c1, k0, k1, weight_sum, image_real, image_complex, flags, st, true);
 }
@@ -1050,7 +1054,8 @@ rick_status model_fft_impl(rick_plan* P, const float* image, int c0, int c1, int
                                  "fused model / row kernel");
     if (s == RICK_OK)
         s = check_launch(launch_fft_columns(reinterpret_cast<float2*>(grids), (int64_t)(c1 - c0) * (k1 - k0),
-                                            P->Ng, false, P->d_twid, occ, st, &launches),
+                                            P->Ng, false, P->d_twid, occ, st, &launches, false,
+                                            (P->Ng - c.N) / 2, (P->Ng + c.N) / 2),
                          "FFT column kernel");
     P->launches += launches;
     return s;
@@ -1149,7 +1154,7 @@ rick_status image_groups_impl(rick_plan* P, float* image_real, float* image_comp
             RK_TRY(grid_impl(P, c0, c1, k0, k1, g, st, P->own_fft));
             RK_TRY(fft_phase_impl(P, g, c0, c1, k0, k1, ws, image_real + (size_t)c0 * NN,
                                   image_complex ? image_complex + 2 * (size_t)c0 * NN : nullptr, st,
-                                  RICK_GRIDDED_BY_PLAN));
+                                  RICK_GRIDDED_BY_PLAN, true));
         }
         if (host_out) {
             // the wait takes the event's latest record, so one event serves every group
@@ -1467,7 +1472,7 @@ rick_status rick_dirty_image_host(rick_plan* plan, const double* uvw, const doub
             const int c0 = (int)((int64_t)c.n_channels * i / nch), c1 = (int)((int64_t)c.n_channels * (i + 1) / nch);
             float* gi = g + (size_t)c0 * plan->planes * plane_floats;
             RK_TRY(fft_phase_impl(plan, gi, c0, c1, 0, plan->planes, d_ws, plan->d_img + (size_t)c0 * NN,
-                                  nullptr, st, RICK_GRIDDED_BY_PLAN));
+                                  nullptr, st, RICK_GRIDDED_BY_PLAN, true));
             RK_CUDA(cudaEventRecord(plan->chunk_done[i], st));
             RK_CUDA(cudaStreamWaitEvent(plan->copy_stream, plan->chunk_done[i], 0));
             RK_CUDA(cudaMemcpyAsync(image_real + (size_t)c0 * NN, plan->d_img + (size_t)c0 * NN,

@@ -3,9 +3,9 @@
 // Eq. 2 needs, per plane, F_k[q][p] = sum_{i,j} G_k[j][i] e^{+2 pi i (i p + j q)/N}
 // (unnormalised); the prediction needs the same with e^{-...}.  The 2-D DFT is
 // a length-N DFT down every column followed by one along every row:
-//   pass 1 (k_fft_columns): one CTA transforms COLS adjacent columns of a plane,
-//     each warp reading and writing rows of COLS x 8 bytes straight from and to
-//     registers;
+//   pass 1, N <= 8192 (k_cols_pair, rick_cols.cu): pairs of adjacent columns as
+//     the lanes of packed FP32 instructions; N = 16384: one column per CTA
+//     (k_fft_columns) or, for imaging, two four-step passes (k_cols_four);
 //   pass 2 (k_fft_rows): one CTA transforms one row, in place; or, for imaging,
 //     k_rows_phase_reduce: one CTA owns one image row q, transforms that row of
 //     every plane of every channel of the launch, applies the phase screen
@@ -69,419 +69,74 @@
 #include <type_traits>
 #include <vector>
 
+#include "rick_dft.cuh"
 #include "rick_internal.cuh"
 
 namespace rick {
 
 namespace {
 
-// cos(2 pi k / 32) for 0 <= k <= 8, from the values of cos(pi k / 16)
-__host__ __device__ constexpr float quarter32(int k) {
-    return k == 0 ? 1.0f
-         : k == 1 ? 0.98078528040323044913f
-         : k == 2 ? 0.92387953251128675613f
-         : k == 3 ? 0.83146961230254523708f
-         : k == 4 ? 0.70710678118654752440f
-         : k == 5 ? 0.55557023301960222474f
-         : k == 6 ? 0.38268343236508977173f
-         : k == 7 ? 0.19509032201612826785f
-         : 0.0f;
-}
-
-__host__ __device__ constexpr float cos32(int k) {
-    return (k & 31) <= 8    ? quarter32(k & 31)
-         : (k & 31) <= 16 ? -quarter32(16 - (k & 31))
-         : (k & 31) <= 24 ? -quarter32((k & 31) - 16)
-                            : quarter32(32 - (k & 31));
-}
-
-__host__ __device__ constexpr float sin32(int k) { return cos32(k - 8); }
-
-// cos(2 pi k / 64) for 0 <= k <= 16 (cos(pi k / 32), from the FP64 values)
-__host__ __device__ constexpr float quarter64(int k) {
-    return k == 0 ? 1.0f
-         : k == 1 ? 0.99518472667219692873f
-         : k == 2 ? 0.98078528040323043058f
-         : k == 3 ? 0.95694033573220882438f
-         : k == 4 ? 0.92387953251128673848f
-         : k == 5 ? 0.88192126434835504956f
-         : k == 6 ? 0.83146961230254523567f
-         : k == 7 ? 0.77301045336273699338f
-         : k == 8 ? 0.70710678118654757274f
-         : k == 9 ? 0.63439328416364548779f
-         : k == 10 ? 0.55557023301960228867f
-         : k == 11 ? 0.47139673682599780857f
-         : k == 12 ? 0.38268343236508983729f
-         : k == 13 ? 0.29028467725446233105f
-         : k == 14 ? 0.19509032201612833135f
-         : k == 15 ? 0.09801714032956077016f
-         : 0.0f;
-}
-
-__host__ __device__ constexpr float cos64(int k) {
-    return (k & 63) <= 16   ? quarter64(k & 63)
-         : (k & 63) <= 32 ? -quarter64(32 - (k & 63))
-         : (k & 63) <= 48 ? -quarter64((k & 63) - 32)
-                            : quarter64(64 - (k & 63));
-}
-
-__host__ __device__ constexpr float sin64(int k) { return cos64(k - 16); }
-
-// Complex add and subtract as one packed two-lane FP32 instruction each
-// (add/sub.rn.f32x2, sm_100 and later): the same IEEE round-to-nearest results
-// as two scalar instructions, half the issue slots -- the butterflies are
-// mostly adds, and the transform kernels are issue-bound.
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) {
-    uint64_t ra = *reinterpret_cast<uint64_t*>(&a), rb = *reinterpret_cast<uint64_t*>(&b), rd;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
-    return *reinterpret_cast<float2*>(&rd);
-}
-__device__ __forceinline__ float2 csub(float2 a, float2 b) {
-    uint64_t ra = *reinterpret_cast<uint64_t*>(&a), rb = *reinterpret_cast<uint64_t*>(&b), rd;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
-    return *reinterpret_cast<float2*>(&rd);
-}
-__device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
-    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
-// a * (s i), s = +1 (INV) or -1
-template <bool INV>
-__device__ __forceinline__ float2 mul_si(float2 a) {
-    return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
-}
-
-// v * e^(s 2 pi i e / R) for compile-time e and R <= 32 (after unrolling), s = +1 (INV) or -1
-template <bool INV>
-__device__ __forceinline__ float2 twiddle_const(float2 v, int e, int R) {
-    const int k = (e * (32 / R)) & 31;   // in 32nds of a turn
-    if (k == 0) return v;
-    if (k == 8) return mul_si<INV>(v);
-    if (k == 16) return make_float2(-v.x, -v.y);
-    if (k == 24) return mul_si<!INV>(v);
-    const float c = cos32(k), s = INV ? sin32(k) : -sin32(k);
-    return make_float2(fmaf(v.x, c, -v.y * s), fmaf(v.x, s, v.y * c));
-}
-
-// v * e^(s 2 pi i k / 64) for compile-time k (after unrolling), s = +1 (INV) or -1
-template <bool INV>
-__device__ __forceinline__ float2 twiddle64(float2 v, int k) {
-    k &= 63;
-    if (k == 0) return v;
-    if (k == 16) return mul_si<INV>(v);
-    if (k == 32) return make_float2(-v.x, -v.y);
-    if (k == 48) return mul_si<!INV>(v);
-    const float c = cos64(k), s = INV ? sin64(k) : -sin64(k);
-    return make_float2(fmaf(v.x, c, -v.y * s), fmaf(v.x, s, v.y * c));
-}
-
-// In-register length-R DFT, X[f] = sum_t a[t] e^(s 2 pi i t f / R), natural order.
-template <int R, bool INV>
-struct Dft;
-
-template <bool INV>
-struct Dft<2, INV> {
-    static __device__ __forceinline__ void run(float2* a) {
-        const float2 x = a[0], y = a[1];
-        a[0] = cadd(x, y);
-        a[1] = csub(x, y);
-    }
-};
-
-template <bool INV>
-struct Dft<4, INV> {
-    static __device__ __forceinline__ void run(float2* a) {
-        const float2 t0 = cadd(a[0], a[2]), t1 = csub(a[0], a[2]);
-        const float2 t2 = cadd(a[1], a[3]), t3 = mul_si<INV>(csub(a[1], a[3]));
-        a[0] = cadd(t0, t2);
-        a[2] = csub(t0, t2);
-        a[1] = cadd(t1, t3);
-        a[3] = csub(t1, t3);
-    }
-};
-
-// R = 4 S: X[f0 + 4 f1] = sum_{t1 < S} W_S^(t1 f1) [W_R^(t1 f0) sum_{t2 < 4} a[t1 + S t2] W_4^(t2 f0)]
-template <int R, bool INV>
-struct Dft {
-    static_assert(R == 8 || R == 16 || R == 32, "radix");
-    static constexpr int S = R / 4;
-    static __device__ __forceinline__ void run(float2* a) {
-        float2 y[R];  // y[f0 S + t1]
-#pragma unroll
-        for (int t1 = 0; t1 < S; ++t1) {
-            float2 b[4] = {a[t1], a[t1 + S], a[t1 + 2 * S], a[t1 + 3 * S]};
-            Dft<4, INV>::run(b);
-#pragma unroll
-            for (int f0 = 0; f0 < 4; ++f0) y[f0 * S + t1] = twiddle_const<INV>(b[f0], t1 * f0, R);
-        }
-#pragma unroll
-        for (int f0 = 0; f0 < 4; ++f0) {
-            Dft<S, INV>::run(y + f0 * S);
-#pragma unroll
-            for (int f1 = 0; f1 < S; ++f1) a[f0 + 4 * f1] = y[f0 * S + f1];
-        }
-    }
-};
-
-__device__ __forceinline__ int skew(int a) { return a + (a >> 4); }
-// skew(a + 16 k) = skew(a) + 17 k: an offset that is a multiple of 16 becomes
-// a constant added to the skewed base, so unrolled accesses at base + 16 k
-// need no address arithmetic of their own
-__host__ __device__ constexpr int skew16(int k16) { return k16 + k16 / 16; }
-
-template <int LOG2N>
-struct Shape {
-    static constexpr int N = 1 << LOG2N;
-    static constexpr int T = N / 16;                 // threads per transform
-    static constexpr int kR16 = LOG2N / 4;            // radix-16 stages
-    static constexpr int kLastR = 1 << (LOG2N % 4);   // 1: the last stage is radix 16
-    static constexpr int kArray = N + N / 16;         // skewed array length
-    // radix-16 stages with twiddles (all but a last radix-16 stage)
-    static constexpr int kTwStages = kLastR == 1 ? kR16 - 1 : kR16;
-    // butterfly groups t1 of stage s, table entries per t1 (stage 0: 4 powers,
-    // the others: all 15), and the offset of the stage's table
-    __host__ __device__ static constexpr int stage_cnt(int s) { return (N / 16) >> (4 * s); }
-    __host__ __device__ static constexpr int stage_per(int s) { return s == 0 ? 4 : 15; }
-    __host__ __device__ static constexpr int stage_off(int s) {
-        int o = 0;
-        for (int i = 0; i < s; ++i) o += stage_per(i) * stage_cnt(i);
-        return o;
-    }
-    static constexpr int kTw = stage_off(kTwStages);  // twiddle table entries
-    // 128 (LOG2N = 7) only for the four-step column pass at N = 16384
-    static_assert(LOG2N >= 7 && LOG2N <= 14, "128 <= N <= 16384");
-};
-
-// Radix-16 stage s (M = 16^s, not the last stage): a holds the butterfly's
-// inputs u + (N/16) t2 for u = b; the DFT, the twiddles W_N^(t1 f0 M) from the
-// stage's table sw (stage 0: sw[j cnt + t1] = W^(2^j t1 M), j < 4, the other
-// powers formed from them; later stages, whose t1 takes few values, hold all
-// fifteen: sw[(f0 - 1) cnt + t1] = W^(t1 f0 M)) and the stores t1 16 M + g +
-// M f0 into buf.
-template <int LOG2N, bool INV>
-__device__ __forceinline__ void radix16_out(float2 (&a)[16], int b, int s, float2* buf,
-                                            const float2* tw) {
-    using Sh = Shape<LOG2N>;
-    Dft<16, INV>::run(a);
-    const int log2M = 4 * s;
-    const int M = 1 << log2M;
-    const int t1 = b >> log2M, g = b & (M - 1);
-    const int base = (t1 << (log2M + 4)) + g;
-    // output f0 goes to base + M f0: for M >= 16 (M f0 a multiple of 16) and
-    // for M = 1 (base a multiple of 16, f0 < 16) its skewed index is
-    // skew(base) plus a constant
-    float2* out = buf + skew(base);
-    auto at = [&](int f0) -> float2& { return M == 1 ? out[f0] : out[skew16(M * f0)]; };
-    // t1 = 0: the table holds W^0 = 1 exactly, and a * 1 = a exactly
-    const int cnt = Sh::stage_cnt(s);
-    const float2* sw = tw + Sh::stage_off(s) + t1;
-    if (Sh::stage_per(s) == 15) {
-        at(0) = a[0];
-#pragma unroll
-        for (int f0 = 1; f0 < 16; ++f0) {
-            float2 w = sw[(f0 - 1) * cnt];
-            if (!INV) w.y = -w.y;
-            at(f0) = cmulf(a[f0], w);
-        }
-        return;
-    }
-    float2 w[16];
-    w[1] = sw[0];
-    w[2] = sw[cnt];
-    w[4] = sw[2 * cnt];
-    w[8] = sw[3 * cnt];
-    if (!INV) {
-        w[1].y = -w[1].y;
-        w[2].y = -w[2].y;
-        w[4].y = -w[4].y;
-        w[8].y = -w[8].y;
-    }
-    w[3] = cmulf(w[2], w[1]);
-    w[5] = cmulf(w[4], w[1]);
-    w[6] = cmulf(w[4], w[2]);
-    w[7] = cmulf(w[4], w[3]);
-#pragma unroll
-    for (int f0 = 9; f0 < 16; ++f0) w[f0] = cmulf(w[8], w[f0 - 8]);
-    at(0) = a[0];
-#pragma unroll
-    for (int f0 = 1; f0 < 16; ++f0) at(f0) = cmulf(a[f0], w[f0]);
-}
-
-// Stage 0 (M = 1) of the inverse transform whose 16 inputs of thread b all
-// carry one more factor sc (the split row pass's e^(+2 pi i r b / N)): the
-// factor is moved past the butterfly, so output f0 is multiplied by
-// sc W^(b f0) -- the products formed from sc and the stage's four table
-// powers -- instead of every input by sc (31 complex multiplies instead of 42).
-template <int LOG2N>
-__device__ __forceinline__ void radix16_first_scaled(float2 (&a)[16], int b, float2* buf, const float2* tw,
-                                                     float2 sc) {
-    using Sh = Shape<LOG2N>;
-    Dft<16, true>::run(a);
-    const int cnt = Sh::stage_cnt(0);
-    const float2* sw = tw + Sh::stage_off(0) + b;   // t1 = b
-    const float2 w1 = sw[0], w2 = sw[cnt], w4 = sw[2 * cnt], w8 = sw[3 * cnt];
-    float2 w[16];
-    w[0] = sc;
-    w[1] = cmulf(sc, w1);
-    w[2] = cmulf(sc, w2);
-    w[3] = cmulf(w[1], w2);
-    w[4] = cmulf(sc, w4);
-#pragma unroll
-    for (int f0 = 5; f0 < 8; ++f0) w[f0] = cmulf(w[f0 - 4], w4);
-    w[8] = cmulf(sc, w8);
-#pragma unroll
-    for (int f0 = 9; f0 < 16; ++f0) w[f0] = cmulf(w[f0 - 8], w8);
-    float2* out = buf + skew(16 * b);   // outputs 16 b + f0
-#pragma unroll
-    for (int f0 = 0; f0 < 16; ++f0) out[f0] = cmulf(a[f0], w[f0]);
-}
-
-// The middle radix-16 stages (all but the first, which starts from registers,
-// and the last) on buf, in place: loads, barrier, compute and stores, barrier.
-template <int LOG2N, bool INV>
-__device__ __forceinline__ void middle_stages(float2* buf, int b, const float2* tw) {
-    using Sh = Shape<LOG2N>;
-    constexpr int kMiddle = Sh::kTwStages - 1;
-    const float2* in = buf + skew(b);   // inputs b + T t2, T a multiple of 16
-#pragma unroll
-    for (int s = 1; s <= kMiddle; ++s) {
-        float2 a[16];
-#pragma unroll
-        for (int t2 = 0; t2 < 16; ++t2) a[t2] = in[skew16(Sh::T * t2)];
-        __syncthreads();
-        radix16_out<LOG2N, INV>(a, b, s, buf, tw);
-        __syncthreads();
-    }
-}
-
-// The last stage (radix kLastR, or 16), M = N/R, no twiddles: x[j] = X[b + (N/16) j].
-template <int LOG2N, bool INV>
-__device__ __forceinline__ void last_stage(const float2* buf, int b, float2 (&x)[16]) {
-    using Sh = Shape<LOG2N>;
-    constexpr int R = Sh::kLastR == 1 ? 16 : Sh::kLastR;
-    constexpr int NB = 16 / R;          // butterflies per thread
-    constexpr int M = Sh::N / R;
-    const float2* in = buf + skew(b);   // T i + M t2 is a multiple of 16
-#pragma unroll
-    for (int i = 0; i < NB; ++i) {
-        float2 a[R];
-#pragma unroll
-        for (int t2 = 0; t2 < R; ++t2) a[t2] = in[skew16(Sh::T * i + M * t2)];
-        Dft<R, INV>::run(a);
-        // output u + M f0 = b + T (i + NB f0)
-#pragma unroll
-        for (int f0 = 0; f0 < R; ++f0) x[i + NB * f0] = a[f0];
-    }
-}
-
-// One whole transform of the array whose first stage inputs a[t2] = x[b + T t2]
-// are in registers; on return x[j] = X[b + T j].  buf is free on entry and
-// holds the last stage's input on return (a barrier is needed before reuse).
-template <int LOG2N, bool INV>
-__device__ __forceinline__ void transform(float2 (&a)[16], float2* buf, int b, const float2* tw,
-                                          float2 (&x)[16]) {
-    radix16_out<LOG2N, INV>(a, b, 0, buf, tw);
-    __syncthreads();
-    middle_stages<LOG2N, INV>(buf, b, tw);
-    last_stage<LOG2N, INV>(buf, b, x);
-}
-
-template <int LOG2N>
-__device__ __forceinline__ void load_tables(const float2* __restrict__ twid, float2* tw, int tid, int nthreads) {
-    for (int i = tid; i < Shape<LOG2N>::kTw; i += nthreads) tw[i] = __ldg(twid + i);
-}
-
 // ---- pass 1: columns ----------------------------------------------------------
 
-// COLS adjacent columns of one plane per CTA (COLS * N/16 threads), the
-// threads of a column interleaved: thread (b, c) = COLS b + c, so a warp holds
-// COLS columns x 32/COLS butterflies.  The first stage's inputs b + (N/16) t2
-// are read straight into registers and the last stage's outputs written
-// straight back: each warp access covers 32/COLS rows of COLS * 8 bytes (whole
-// 32-byte sectors for COLS = 4), with no staging through shared memory.  Column
-// c's skewed array is offset by 32/COLS banks from column c - 1's, so the
-// COLS arrays a half-warp touches in every stage fall on distinct banks.
-template <int LOG2N, int COLS, bool INV>
-__global__ void __launch_bounds__(COLS * (1 << LOG2N) / 16)
-k_fft_columns(float2* __restrict__ grids, const float2* __restrict__ twid, Occupancy occ, int64_t plane0) {
+// N = 16384, outside the imaging calls with tiles of 32 or more: one column of
+// one plane per CTA (blockIdx.x, blockIdx.y), straight from and to registers.
+template <int LOG2N, bool INV>
+__global__ void __launch_bounds__((1 << LOG2N) / 16)
+k_fft_columns(float2* __restrict__ grids, const float2* __restrict__ twid) {
     using Sh = Shape<LOG2N>;
     constexpr int N = Sh::N, T = Sh::T;
-    constexpr int kStride = Sh::kArray + 16 / COLS;   // float2 per column array
-    __shared__ uint8_t s_live[N / 16];
-    const int64_t pl = plane0 + blockIdx.y;
-    const int tcol = (int)(blockIdx.x * COLS) >> occ.tshift;
-    if (occ.col != nullptr && occ.col[pl * occ.NT + tcol] == 0) return;
-    constexpr int kThreads = COLS * T;
     extern __shared__ __align__(16) float2 fsm[];
     float2* tw = fsm;
-    const int tid = threadIdx.x;
-    const int c = tid % COLS, b = tid / COLS;
-    float2* buf = fsm + Sh::kTw + c * kStride;
-    float2* col = grids + (size_t)blockIdx.y * N * N + (size_t)blockIdx.x * COLS + c;
-    load_tables<LOG2N>(twid, tw, tid, kThreads);
-    if (occ.tile != nullptr)
-        for (int ty = tid; ty < occ.NT; ty += kThreads)
-            s_live[ty] = (uint8_t)((occ.tile[(pl * occ.NT + ty) * occ.words + (tcol >> 5)] >> (tcol & 31)) & 1u);
+    float2* buf = fsm + Sh::kTw;
+    const int b = threadIdx.x;
+    float2* col = grids + (size_t)blockIdx.y * N * N + (size_t)blockIdx.x;
+    load_tables<LOG2N>(twid, tw, b, T);
     __syncthreads();
-    const bool in_mask = occ.tile != nullptr && !occ.tiles_out, out_mask = occ.tile != nullptr && occ.tiles_out;
     float2 a[16], x[16];
 #pragma unroll
-    for (int t2 = 0; t2 < 16; ++t2) {
-        const int row = b + T * t2;
-        // an unreached tile is zero (and possibly unwritten): not read
-        a[t2] = (!in_mask || s_live[row >> occ.tshift]) ? __ldcs(col + (size_t)row * N) : make_float2(0.f, 0.f);
-    }
+    for (int t2 = 0; t2 < 16; ++t2) a[t2] = __ldcs(col + (size_t)(b + T * t2) * N);
     transform<LOG2N, INV>(a, buf, b, tw, x);
-    // with tiles_out, only the reached tiles of the result are written
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        const int row = b + T * j;
-        if (!out_mask || s_live[row >> occ.tshift]) __stcs(col + (size_t)row * N, x[j]);
-    }
+    for (int j = 0; j < 16; ++j) __stcs(col + (size_t)(b + T * j) * N, x[j]);
 }
 
-// The column pass over the reached tile columns only (occ.list): a persistent
-// CTA (one or two per SM) loads the twiddle tables once, then takes COLS
-// adjacent columns at a time from the list -- tile column entry e = p NT + tx
-// gives columns (tx << tshift) + COLS j of plane p -- with an atomic work
-// counter, and transforms them as k_fft_columns does.  The unreached tile
-// columns cost nothing: with one CTA per column most CTAs of a sparse launch
-// only looked up their mask byte and exited, and at N = 16384 (180 KB of
-// shared memory, one CTA per SM at a time) those empty CTAs took most of the
-// pass.
-template <int LOG2N, int COLS, bool INV>
-__global__ void __launch_bounds__(COLS * (1 << LOG2N) / 16)
+// The same over the reached tile columns only (occ.list): a persistent CTA
+// loads the twiddle tables once, then takes one column at a time from the list
+// -- tile column entry e = p NT + tx gives columns (tx << tshift) + j of plane
+// p -- with an atomic work counter.  With one CTA per column most CTAs of a
+// sparse launch only looked up their mask byte and exited (180 KB of shared
+// memory, one CTA per SM at a time), which took most of the pass.
+template <int LOG2N, bool INV>
+__global__ void __launch_bounds__((1 << LOG2N) / 16)
 k_fft_columns_list(float2* __restrict__ grids, const float2* __restrict__ twid, Occupancy occ) {
     using Sh = Shape<LOG2N>;
     constexpr int N = Sh::N, T = Sh::T;
-    constexpr int kStride = Sh::kArray + 16 / COLS;
-    constexpr int kThreads = COLS * T;
     __shared__ uint8_t s_live[N / 16];
     __shared__ uint32_t s_item;
     extern __shared__ __align__(16) float2 fsm[];
     float2* tw = fsm;
-    const int tid = threadIdx.x;
-    const int c = tid % COLS, b = tid / COLS;
-    float2* buf = fsm + Sh::kTw + c * kStride;
-    load_tables<LOG2N>(twid, tw, tid, kThreads);
-    const uint32_t per = (1u << occ.tshift) / COLS;          // CTA items per tile column
+    float2* buf = fsm + Sh::kTw;
+    const int b = threadIdx.x;
+    load_tables<LOG2N>(twid, tw, b, T);
+    const uint32_t per = 1u << occ.tshift;                   // CTA items per tile column
     const uint64_t total = (uint64_t)__ldg(occ.list) * per;
     const bool in_mask = !occ.tiles_out, out_mask = occ.tiles_out;
     // thread 0 takes the next item while the current one is transformed
-    uint32_t next = tid == 0 ? atomicAdd(occ.list + 1, 1u) : 0u;
+    uint32_t next = b == 0 ? atomicAdd(occ.list + 1, 1u) : 0u;
     for (;;) {
-        if (tid == 0) s_item = next;
+        if (b == 0) s_item = next;
         __syncthreads();   // also: the previous item's last stage has read buf
         const uint32_t item = s_item;
         if (item >= total) break;
-        if (tid == 0) next = atomicAdd(occ.list + 1, 1u);
+        if (b == 0) next = atomicAdd(occ.list + 1, 1u);
         const uint32_t e = __ldg(occ.list + 2 + item / per);
         const int64_t pl = e / (uint32_t)occ.NT;
         const int tcol = (int)(e - (uint32_t)pl * occ.NT);
-        const int x0 = (tcol << occ.tshift) + (int)(item % per) * COLS;
-        for (int ty = tid; ty < occ.NT; ty += kThreads)
+        const int x0 = (tcol << occ.tshift) + (int)(item % per);
+        for (int ty = b; ty < occ.NT; ty += T)
             s_live[ty] = (uint8_t)((occ.tile[(pl * occ.NT + ty) * occ.words + (tcol >> 5)] >> (tcol & 31)) & 1u);
         __syncthreads();
-        float2* col = grids + (size_t)pl * N * N + x0 + c;
+        float2* col = grids + (size_t)pl * N * N + x0;
         float2 a[16], x[16];
 #pragma unroll
         for (int t2 = 0; t2 < 16; ++t2) {
@@ -1130,11 +785,12 @@ k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __rest
     float2* buf = fsm + Sh::kTw;
     float2* zrot = buf + Sh::kArray;                            // z = e^(-2 pi i dt) per pixel
     float* js = reinterpret_cast<float*>(zrot + N);             // J_c(p) times the pixel's scale
-    // mesh row q (blockIdx.x) is image row q - off and mesh pixel pm image
+    // image row qi (blockIdx.x) is mesh row qi + off and mesh pixel pm image
     // pixel pm - off (a padded mesh holds the image in its central Ni x Ni;
     // the model is zero elsewhere)
+    // (the rows of the padding are zero: not written, the column pass does not read them)
     const int Ni = P.Ni, off = P.off;
-    const int b = threadIdx.x, q = blockIdx.x, qi = q - off;
+    const int b = threadIdx.x, qi = blockIdx.x, q = qi + off;
     const size_t NN = (size_t)N * N, NNi = (size_t)Ni * Ni;
     const bool warp_mask = occ.tshift >= 5 && T >= 32;
     const int lane = b & 31;
@@ -1155,18 +811,6 @@ k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __rest
         }
         return live;
     };
-    if ((unsigned)qi >= (unsigned)Ni) {
-        // a row of the padding: its transform is zero, written where it is read
-        for (int r = 0; r < P.nc * P.nk; ++r) {
-            if (occ.plane != nullptr && occ.plane[r] == 0) continue;
-            const uint32_t live = live_cols(r);
-            float2* row = grids + (size_t)r * NN + (size_t)q * N;
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-                if ((live >> j) & 1u) __stcs(row + b + T * j, make_float2(0.f, 0.f));
-        }
-        return;
-    }
     const uint2* turns = pix_turns + (size_t)qi * Ni;
     load_tables<LOG2N>(twid, tw, b, T);
 #pragma unroll 4
@@ -1235,11 +879,6 @@ k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __rest
         }
     }
 }
-
-// columns per CTA in pass 1: warp accesses of 32-byte row pieces (whole DRAM
-// sectors) where 4 N/16 threads fit a CTA, else 16 bytes
-template <int LOG2N>
-constexpr int kCols = LOG2N <= 12 ? 4 : LOG2N == 13 ? 2 : 1;
 
 // Occupancy of the planes p = cc nk + kk of the launch from the bin offsets:
 // one thread per tile (tx fastest), reached iff tile_reach() > 0 -- the
@@ -1319,42 +958,48 @@ cudaError_t columns_four(float2* grids, int64_t n_planes, const float2* t4, cons
 
 template <int LOG2N, bool INV>
 cudaError_t columns_one(float2* grids, int64_t n_planes, const float2* twid, const Occupancy& occ,
-                        cudaStream_t st, bool fourstep = false) {
+                        cudaStream_t st, bool fourstep = false, int row_lo = 0, int row_hi = 1 << LOG2N) {
     using Sh = Shape<LOG2N>;
-    constexpr int cols = kCols<LOG2N>;
-    if (LOG2N == 14 && fourstep) {
-        // every (group, n1) and (group, k2) item index below 2^32
-        if ((uint64_t)n_planes * 16384u * kFourL / 32u >= (1ull << 32)) return cudaErrorInvalidValue;
-        const float2* t4 = twid + Shape<14>::kTw + Shape<12>::kTw + 4 * 256 + 256;
-        return occ.list != nullptr && occ.tile != nullptr ? columns_four<INV, true>(grids, n_planes, t4, occ, st)
-                                                          : columns_four<INV, false>(grids, n_planes, t4, occ, st);
-    }
-    const size_t smem = (size_t)(Sh::kTw + cols * (Sh::kArray + 16 / cols)) * sizeof(float2);
-    if (occ.list != nullptr && occ.tile != nullptr) {
-        // persistent CTAs over the listed tile columns; the work counter
-        // list[1] starts at zero for every pass
-        auto fl = k_fft_columns_list<LOG2N, cols, INV>;
-        cudaError_t e = cudaFuncSetAttribute(fl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if constexpr (LOG2N < 14) {
+        // the pair kernel's tables follow the stage tables and the 256 phasors
+        return launch_cols_pair(grids, n_planes, Sh::N, INV, twid + Sh::kTw + 256, occ, row_lo, row_hi, st);
+    } else {
+
+        if (fourstep) {
+            // every (group, n1) and (group, k2) item index below 2^32
+            if ((uint64_t)n_planes * 16384u * kFourL / 32u >= (1ull << 32)) return cudaErrorInvalidValue;
+            const float2* t4 = twid + Shape<14>::kTw + Shape<12>::kTw + 4 * 256 + 256;
+            return occ.list != nullptr && occ.tile != nullptr
+                       ? columns_four<INV, true>(grids, n_planes, t4, occ, st)
+                       : columns_four<INV, false>(grids, n_planes, t4, occ, st);
+        }
+        const size_t smem = (size_t)(Sh::kTw + Sh::kArray + 16) * sizeof(float2);
+        if (occ.list != nullptr && occ.tile != nullptr) {
+            // persistent CTAs over the listed tile columns; the work counter
+            // list[1] starts at zero for every pass
+            auto fl = k_fft_columns_list<LOG2N, INV>;
+            cudaError_t e = cudaFuncSetAttribute(fl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            int per_sm = 0, dev = 0, sms = 0;
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fl, Sh::T, smem)) != cudaSuccess)
+                return e;
+            if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+            if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+            if (per_sm < 1) return cudaErrorInvalidConfiguration;
+            if ((e = cudaMemsetAsync(occ.list + 1, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
+            fl<<<(unsigned)(per_sm * sms), Sh::T, smem, st>>>(grids, twid, occ);
+            return cudaGetLastError();
+        }
+        auto fn = k_fft_columns<LOG2N, INV>;
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        int per_sm = 0, dev = 0, sms = 0;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fl, cols * Sh::T, smem)) != cudaSuccess)
-            return e;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        if ((e = cudaMemsetAsync(occ.list + 1, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
-        fl<<<(unsigned)(per_sm * sms), cols * Sh::T, smem, st>>>(grids, twid, occ);
-        return cudaGetLastError();
+        for (int64_t p0 = 0; p0 < n_planes; p0 += 65535) {
+            const unsigned np = (unsigned)(n_planes - p0 < 65535 ? n_planes - p0 : 65535);
+            fn<<<dim3(Sh::N, np), Sh::T, smem, st>>>(grids + p0 * Sh::N * Sh::N, twid);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
+        return cudaSuccess;
     }
-    auto fn = k_fft_columns<LOG2N, cols, INV>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    for (int64_t p0 = 0; p0 < n_planes; p0 += 65535) {
-        const unsigned np = (unsigned)(n_planes - p0 < 65535 ? n_planes - p0 : 65535);
-        fn<<<dim3(Sh::N / cols, np), cols * Sh::T, smem, st>>>(grids + p0 * Sh::N * Sh::N, twid, occ, p0);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    return cudaSuccess;
 }
 
 template <int LOG2N, bool INV>
@@ -1465,10 +1110,28 @@ void append_twiddles(int N, std::vector<float2>& out) {
     }
 }
 
+// The tables of k_cols_pair (PairShape): per part s of SPLIT (2 for N = 8192)
+// e^(+2 pi i b (s + SPLIT f0) / N) at [s][f0][b], f0 < 16, b < M / 16, then the
+// later stages of the M-point transform (M = N / SPLIT).
+void append_pair_tables(int N, std::vector<float2>& out) {
+    const int split = N == 8192 ? 2 : 1, M = N / split;
+    const double two_pi = 6.283185307179586476925;
+    for (int s = 0; s < split; ++s)
+        for (int f0 = 0; f0 < 16; ++f0)
+            for (int b = 0; b < M / 16; ++b) {
+                const double a = two_pi * (double)((int64_t)b * (s + split * f0) % N) / N;
+                out.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
+            }
+    std::vector<float2> stages;
+    append_twiddles(M, stages);
+    out.insert(out.end(), stages.begin() + 4 * (M / 16), stages.end());
+}
+
 }  // namespace
 
 void fft_twiddles(int N, std::vector<float2>& out) {
-    // N < 16384: the stage tables, then e^(2 pi i j / 256), j < 256.
+    // N < 16384: the stage tables, then e^(2 pi i j / 256), j < 256, then the
+    // column pass's tables (append_pair_tables).
     // N = 16384: the 4096-point tables of the split fused row pass follow,
     // then its split twiddles [r T + b] = e^(+2 pi i r b / N), r < 4, b < T = 256,
     // then e^(2 pi i j / 256), j < 256, then the four-step column pass's tables
@@ -1481,6 +1144,7 @@ void fft_twiddles(int N, std::vector<float2>& out) {
             const double a = 6.283185307179586476925 * (double)j / 256.0;
             out.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
         }
+        append_pair_tables(N, out);
     }
     if (log2_exact(N) == 14) {
         append_twiddles(4096, out);
@@ -1537,13 +1201,14 @@ cudaError_t launch_fft2d(float2* grids, int64_t n_planes, int N, bool inverse, c
 }
 
 cudaError_t launch_fft_columns(float2* grids, int64_t n_planes, int N, bool inverse, const float2* twid,
-                               const Occupancy& occ, cudaStream_t st, int* launches, bool fourstep) {
+                               const Occupancy& occ, cudaStream_t st, int* launches, bool fourstep, int row_lo, int row_hi) {
+    if (row_hi <= 0) row_hi = N;
     if (n_planes <= 0) return cudaSuccess;
     cudaError_t e = cudaErrorInvalidValue;
 #define RICK_FFT_CASE(LG)                                                                   \
     case LG:                                                                                \
-        e = inverse ? columns_one<LG, true>(grids, n_planes, twid, occ, st, fourstep)       \
-                    : columns_one<LG, false>(grids, n_planes, twid, occ, st, fourstep);     \
+        e = inverse ? columns_one<LG, true>(grids, n_planes, twid, occ, st, fourstep, row_lo, row_hi)   \
+                    : columns_one<LG, false>(grids, n_planes, twid, occ, st, fourstep, row_lo, row_hi); \
         break;
     switch (log2_exact(N)) {
         RICK_FFT_CASE(8)
@@ -1595,7 +1260,7 @@ cudaError_t launch_model_rows(const PhaseParams& P, const float* image, const ui
         const size_t smem = (size_t)(Sh::kTw + Sh::kArray + Sh::N) * sizeof(float2) + (size_t)Sh::N * sizeof(float); \
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);      \
         if (e == cudaSuccess) {                                                                     \
-            fn<<<Sh::N, Sh::T, smem, st>>>(P, image, pix_turns, pix_model_scale, twid, grids, occ); \
+            fn<<<P.Ni, Sh::T, smem, st>>>(P, image, pix_turns, pix_model_scale, twid, grids, occ); \
             e = cudaGetLastError();                                                                 \
         }                                                                                           \
         break;                                                                                      \

@@ -292,9 +292,14 @@ cudaError_t launch_occupancy(const uint32_t* offsets, int c0, int nc, int k0, in
 // fourstep (N = 16384 only): the two four-step passes, which leave the rows
 // of every plane in the four-step order (mesh row m at row 128 (m mod 128) +
 // m / 128), the order the fused row pass reads with PhaseParams::rows_four.
+// [row_lo, row_hi) (N <= 8192; 0, 0: all rows): the only rows the inverse
+// transform stores; the rows outside are zero for the forward transform.
 cudaError_t launch_fft_columns(float2* grids, int64_t n_planes, int N, bool inverse, const float2* twid,
                                const Occupancy& occ, cudaStream_t stream, int* launches,
-                               bool fourstep = false);
+                               bool fourstep = false, int row_lo = 0, int row_hi = 0);
+// The column pass at N <= 8192 (rick_cols.cu); table: the pair kernel's tables of the plan.
+cudaError_t launch_cols_pair(float2* grids, int64_t n_planes, int N, bool inverse, const float2* table,
+                             const Occupancy& occ, int row_lo, int row_hi, cudaStream_t stream);
 // Pass 2 fused with the phase screen and reduction: grids must hold the
 // column-transformed planes [nc][nk][N][N]; image_real [nc][N][N] (+=).
 // With occ, unreached planes are skipped and unreached tile columns read as

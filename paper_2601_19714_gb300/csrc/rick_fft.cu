@@ -330,37 +330,58 @@ __global__ void k_pixel_phase(PhaseParams P, const float* __restrict__ inv_taper
 // The per-pixel turns and scale come from the plan's table (k_pixel_phase).
 // The next row is loaded into registers while the current one is transformed.
 // Two CTAs per SM for N <= 4096 (at most 128 registers).
+// CTAs an SM that the fused row passes are compiled for: 16 warps, i.e. at most
+// 128 registers a thread (with the two CTAs of N = 4096 asked for at every
+// length, N = 2048 took 172 registers and ran 8 warps an SM: with the crop 264 ->
+// 122 us on 4 channels x 8 planes of a 2048^2 mesh; N = 256's 16 threads take a
+// whole warp's registers, so 16 CTAs are as many as 128 registers allow)
+constexpr int row_min_ctas(int log2n) { return log2n >= 13 ? 1 : log2n >= 9 ? (1 << (13 - log2n)) : 16; }
 constexpr int kHornerBlock = 8;   // planes per Horner block of the fused row pass
 
-template <int LOG2N, bool COMPLEX_OUT, bool PADDED>
-__global__ void __launch_bounds__((1 << LOG2N) / 16, LOG2N <= 12 ? 2 : 1)
+// The mesh pixels b + T j, j < 16, of a thread that a row pass keeps: all (PAD =
+// 0), the middle eight of a mesh twice the image (PAD = 1: exactly the image's),
+// or the middle four (PAD = 2: every padding by 4 or more, whose image pixels
+// among them are told apart at run time).  Phasing, summing and then dropping the
+// other pixels took a quarter of the pass: rows of a 4096^2 mesh padded by 2
+// (16 channels x 16 planes) 4.37 -> 3.60 ms, of an 8192^2 one (6 x 20) 14.4 ->
+// 11.9 ms.
+template <int PAD>
+struct Crop {
+    static constexpr int J0 = PAD == 0 ? 0 : PAD == 1 ? 4 : 6;
+    static constexpr int NJ = PAD == 0 ? 16 : PAD == 1 ? 8 : 4;
+    static constexpr bool kExact = PAD < 2;
+};
+
+template <int LOG2N, bool COMPLEX_OUT, int PAD>
+__global__ void __launch_bounds__((1 << LOG2N) / 16, row_min_ctas(LOG2N))
 k_rows_phase_reduce(PhaseParams P, const float2* __restrict__ grids, const double* __restrict__ wsum,
                     const uint2* __restrict__ pix_turns, const float* __restrict__ pix_scale,
                     const float2* __restrict__ twid, float* __restrict__ image_real,
                     float2* __restrict__ image_complex, Occupancy occ) {
     using Sh = Shape<LOG2N>;
-    constexpr int N = Sh::N, T = Sh::T;
+    using Cr = Crop<PAD>;
+    constexpr int N = Sh::N, T = Sh::T, J0 = Cr::J0, NJ = Cr::NJ;
     extern __shared__ __align__(16) float2 fsm[];
     float2* tw = fsm;
     float2* buf = fsm + Sh::kTw;
     float2* turn256 = buf + Sh::kArray;                          // e^(2 pi i j / 256)
     float2* zrot = turn256 + 256;                                // z = e^(-2 pi i dt) per pixel
     // the channel's finished blocks per pixel: Re of the phased sums
-    float* part = reinterpret_cast<float*>(zrot + N);
-    // image row q (blockIdx.x) is row q + off of the mesh; mesh pixel pm is
-    // image pixel pm - off (a padded mesh keeps its central Ni x Ni; without
-    // padding, off = 0 and Ni = N at compile time)
-    const int Ni = PADDED ? P.Ni : N, off = PADDED ? P.off : 0;
+    float* part = reinterpret_cast<float*>(zrot + NJ * T);
+    // image row q (blockIdx.x) is row q + off of the mesh; mesh pixel b + T (J0 + j)
+    // is image pixel b + T j + poff (Crop)
+    const int Ni = PAD == 0 ? N : PAD == 1 ? N / 2 : P.Ni, off = PAD == 0 ? 0 : PAD == 1 ? N / 4 : P.off;
+    const int poff = T * J0 - off;
     const int b = threadIdx.x, q = blockIdx.x;
     const float* scl = pix_scale + (size_t)q * Ni;               // per-pixel scale (read once per channel)
     const uint2* turns = pix_turns + (size_t)q * Ni;
     load_tables<LOG2N>(twid, tw, b, T);
     for (int j = b; j < 256; j += T) turn256[j] = __ldg(twid + Sh::kTw + j);
 #pragma unroll 4
-    for (int j = 0; j < 16; ++j) {
-        const int pm = b + T * j, p = pm - off;
+    for (int j = 0; j < NJ; ++j) {
+        const int pm = b + T * j, p = pm + poff;
         float s = 0.f, c = 1.f;
-        if (!PADDED || (unsigned)p < (unsigned)Ni)
+        if (Cr::kExact || (unsigned)p < (unsigned)Ni)
             sincospif((float)(int32_t)__ldg(&turns[p].y) * 4.656612873077392578125e-10f /* 2^-31 */, &s, &c);
         zrot[pm] = make_float2(c, -s);
         if (!COMPLEX_OUT) part[pm] = 0.f;
@@ -407,13 +428,13 @@ k_rows_phase_reduce(PhaseParams P, const float2* __restrict__ grids, const doubl
     if (r < n_rows) load_row(r, a);
     __syncthreads();
     for (int cc = 0; cc < P.nc; ++cc) {
-        float2 acc[16];
+        float2 acc[NJ];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.f, 0.f);
+        for (int j = 0; j < NJ; ++j) acc[j] = make_float2(0.f, 0.f);
         for (int kk = 0; kk < P.nk; ++kk) {
             if (cc * P.nk + kk != r) {   // an unreached plane: F_k = 0
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
+                for (int j = 0; j < NJ; ++j) {
                     const float2 z = zrot[b + T * j];
                     acc[j] = make_float2(fmaf(acc[j].x, z.x, -acc[j].y * z.y), fmaf(acc[j].x, z.y, acc[j].y * z.x));
                 }
@@ -427,10 +448,10 @@ k_rows_phase_reduce(PhaseParams P, const float2* __restrict__ grids, const doubl
                 last_stage<LOG2N, true>(buf, b, x);
                 __syncthreads();   // buf is rewritten by the next row's first stage
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
+                for (int j = 0; j < NJ; ++j) {
                     const float2 z = zrot[b + T * j];
-                    acc[j] = make_float2(fmaf(acc[j].x, z.x, fmaf(-acc[j].y, z.y, x[j].x)),
-                                         fmaf(acc[j].x, z.y, fmaf(acc[j].y, z.x, x[j].y)));
+                    acc[j] = make_float2(fmaf(acc[j].x, z.x, fmaf(-acc[j].y, z.y, x[J0 + j].x)),
+                                         fmaf(acc[j].x, z.y, fmaf(acc[j].y, z.x, x[J0 + j].y)));
                 }
             }
             const bool last = kk == P.nk - 1;
@@ -444,11 +465,11 @@ k_rows_phase_reduce(PhaseParams P, const float2* __restrict__ grids, const doubl
                 inv_ws = ws != 0.0 ? (float)(1.0 / ws) : 0.0f;
             }
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                // pixels outside the image (a padded mesh) are computed from a
+            for (int j = 0; j < NJ; ++j) {
+                // pixels outside the image (inexact crop) are computed from a
                 // valid index and not stored, so that every load is unconditional
-                const int pm = b + T * j, p = pm - off;
-                const bool in_img = !PADDED || (unsigned)p < (unsigned)Ni;
+                const int pm = b + T * j, p = pm + poff;
+                const bool in_img = Cr::kExact || (unsigned)p < (unsigned)Ni;
                 const int pc = in_img ? p : 0;
                 // e^(2 pi i t) for t = tk 2^-32 turns, table-driven: the
                 // nearest 1/256 of a turn from the table, the rest
@@ -513,7 +534,7 @@ k_rows_phase_reduce(PhaseParams P, const float2* __restrict__ grids, const doubl
 // reached plane takes no phasor -- the zeros the unpruned pass computes, so
 // the pruned result is still the unpruned one.  (In the unsplit pass the same
 // change measured 9 % slower at 4096^2 and is not made.)
-template <int LOG2SUB, int SPLIT, bool COMPLEX_OUT, bool PADDED>
+template <int LOG2SUB, int SPLIT, bool COMPLEX_OUT, int PAD>
 __global__ void __launch_bounds__((1 << LOG2SUB) / 16, LOG2SUB <= 12 ? 2 : 1)
 k_rows_phase_reduce_split(PhaseParams P, const float2* __restrict__ grids, const double* __restrict__ wsum,
                           const uint2* __restrict__ pix_turns, const float* __restrict__ pix_scale,
@@ -523,27 +544,28 @@ k_rows_phase_reduce_split(PhaseParams P, const float2* __restrict__ grids, const
     static_assert(SPLIT == 4 && LOG2SUB == 12, "split");
     using Sh = Shape<LOG2SUB>;
     constexpr int M = Sh::N, T = Sh::T;     // sub-transform: points, threads
-    constexpr int N = SPLIT * M;
+    using Cr = Crop<PAD>;
+    constexpr int N = SPLIT * M, J0 = Cr::J0, NJ = Cr::NJ;
     extern __shared__ __align__(16) float2 fsm[];
     float2* tw = fsm;
     float2* buf = fsm + Sh::kTw;
     float2* turn256 = buf + Sh::kArray;                          // e^(2 pi i j / 256)
     float2* zrot = turn256 + 256;                                // z per owned pixel
-    float* part = reinterpret_cast<float*>(zrot + M);
-    // image row q is mesh row q + off; mesh pixel SPLIT k + r is image pixel
-    // SPLIT k + r - off (a padded mesh keeps its central Ni x Ni; without
-    // padding, off = 0 and Ni = N at compile time)
-    const int Ni = PADDED ? P.Ni : N, off = PADDED ? P.off : 0;
+    float* part = reinterpret_cast<float*>(zrot + NJ * T);
+    // image row q is mesh row q + off; mesh pixel SPLIT (b + T (J0 + j)) + r is
+    // image pixel SPLIT (b + T j) + r + poff (Crop)
+    const int Ni = PAD == 0 ? N : PAD == 1 ? N / 2 : P.Ni, off = PAD == 0 ? 0 : PAD == 1 ? N / 4 : P.off;
+    const int poff = SPLIT * T * J0 - off;
     const int b = threadIdx.x, q = blockIdx.x / SPLIT, par = blockIdx.x % SPLIT;
     const float* scl = pix_scale + (size_t)q * Ni;
     const uint2* turns = pix_turns + (size_t)q * Ni;
     load_tables<LOG2SUB>(twid_sub, tw, b, T);
     for (int j = b; j < 256; j += T) turn256[j] = __ldg(twid_sub + Sh::kTw + SPLIT * T + j);
 #pragma unroll 4
-    for (int j = 0; j < 16; ++j) {
-        const int k = b + T * j, p = SPLIT * k + par - off;
+    for (int j = 0; j < NJ; ++j) {
+        const int k = b + T * j, p = SPLIT * k + par + poff;
         float s = 0.f, c = 1.f;
-        if (!PADDED || (unsigned)p < (unsigned)Ni)
+        if (Cr::kExact || (unsigned)p < (unsigned)Ni)
             sincospif((float)(int32_t)__ldg(&turns[p].y) * 4.656612873077392578125e-10f /* 2^-31 */, &s, &c);
         zrot[k] = make_float2(c, -s);
         if (!COMPLEX_OUT) part[k] = 0.f;
@@ -656,9 +678,9 @@ k_rows_phase_reduce_split(PhaseParams P, const float2* __restrict__ grids, const
     if (r < n_rows) load_row(r, a);
     __syncthreads();
     for (int cc = 0; cc < P.nc; ++cc) {
-        float2 acc[16];
+        float2 acc[NJ];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.f, 0.f);
+        for (int j = 0; j < NJ; ++j) acc[j] = make_float2(0.f, 0.f);
         // filled: the current block has a reached plane; any: the channel has
         bool filled = false, any = false;
         for (int kk = 0; kk < P.nk; ++kk) {
@@ -667,7 +689,7 @@ k_rows_phase_reduce_split(PhaseParams P, const float2* __restrict__ grids, const
                 // and stays zero, so there is nothing to rotate
                 if (filled) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
+                    for (int j = 0; j < NJ; ++j) {
                         const float2 z = zrot[b + T * j];
                         acc[j] = make_float2(fmaf(acc[j].x, z.x, -acc[j].y * z.y),
                                              fmaf(acc[j].x, z.y, acc[j].y * z.x));
@@ -689,10 +711,10 @@ k_rows_phase_reduce_split(PhaseParams P, const float2* __restrict__ grids, const
                 last_stage<LOG2SUB, true>(buf, b, x);
                 __syncthreads();   // buf is rewritten by the next row's first stage
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
+                for (int j = 0; j < NJ; ++j) {
                     const float2 z = zrot[b + T * j];
-                    acc[j] = make_float2(fmaf(acc[j].x, z.x, fmaf(-acc[j].y, z.y, x[j].x)),
-                                         fmaf(acc[j].x, z.y, fmaf(acc[j].y, z.x, x[j].y)));
+                    acc[j] = make_float2(fmaf(acc[j].x, z.x, fmaf(-acc[j].y, z.y, x[J0 + j].x)),
+                                         fmaf(acc[j].x, z.y, fmaf(acc[j].y, z.x, x[J0 + j].y)));
                 }
                 filled = any = true;
             }
@@ -710,11 +732,11 @@ k_rows_phase_reduce_split(PhaseParams P, const float2* __restrict__ grids, const
                 inv_ws = ws != 0.0 ? (float)(1.0 / ws) : 0.0f;
             }
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                // pixels outside the image (a padded mesh) are computed from a
+            for (int j = 0; j < NJ; ++j) {
+                // pixels outside the image (inexact crop) are computed from a
                 // valid index and not stored, so that every load is unconditional
-                const int k = b + T * j, p = SPLIT * k + par - off;
-                const bool in_img = !PADDED || (unsigned)p < (unsigned)Ni;
+                const int k = b + T * j, p = SPLIT * k + par + poff;
+                const bool in_img = Cr::kExact || (unsigned)p < (unsigned)Ni;
                 const int pc = in_img ? p : 0;
                 float sn = 0.f, cs = 1.f;   // acc is zero in an empty block
                 if (!empty) {
@@ -774,7 +796,7 @@ k_rows_phase_reduce_split(PhaseParams P, const float2* __restrict__ grids, const
 // reached tile columns are written (the column pass reads nothing else, and
 // the degridder only the reached tiles).
 template <int LOG2N>
-__global__ void __launch_bounds__((1 << LOG2N) / 16, LOG2N <= 12 ? 2 : 1)
+__global__ void __launch_bounds__((1 << LOG2N) / 16, row_min_ctas(LOG2N))
 k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __restrict__ pix_turns,
              const float* __restrict__ pix_model_scale, const float2* __restrict__ twid,
              float2* __restrict__ grids, Occupancy occ) {
@@ -1017,16 +1039,16 @@ cudaError_t rows_one(float2* grids, int64_t n_planes, const float2* twid, cudaSt
     return cudaSuccess;
 }
 
-template <int LOG2N, bool CPLX, bool PADDED>
+template <int LOG2N, bool CPLX, int PAD>
 cudaError_t fused_one(const PhaseParams& P, const float2* grids, const double* wsum, const uint2* pix_turns,
                       const float* pix_scale, const float2* twid, float* image_real, float2* image_complex,
                       const Occupancy& occ, cudaStream_t st) {
     using Sh = Shape<LOG2N>;
-    auto fn = k_rows_phase_reduce<LOG2N, CPLX, PADDED>;
+    auto fn = k_rows_phase_reduce<LOG2N, CPLX, PAD>;
     // tables, the transform array and the 256 phasors, then per pixel z and
     // (real output) the partial sum
     const size_t smem = (size_t)(Sh::kTw + Sh::kArray + 256) * sizeof(float2) +
-                        (size_t)Sh::N * (sizeof(float2) + (CPLX ? 0 : 1) * sizeof(float));
+                        (size_t)Sh::T * Crop<PAD>::NJ * (sizeof(float2) + (CPLX ? 0 : 1) * sizeof(float));
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     fn<<<P.Ni, Sh::T, smem, st>>>(P, grids, wsum, pix_turns, pix_scale, twid, image_real, image_complex, occ);
@@ -1035,15 +1057,15 @@ cudaError_t fused_one(const PhaseParams& P, const float2* grids, const double* w
 
 // N = 16384: four CTAs per image row, each with the 4096-point tables (they
 // follow the 16384-point tables in twid)
-template <bool CPLX, bool PADDED>
+template <bool CPLX, int PAD>
 cudaError_t fused_split(const PhaseParams& P, const float2* grids, const double* wsum, const uint2* pix_turns,
                         const float* pix_scale, const float2* twid, float* image_real, float2* image_complex,
                         const Occupancy& occ, cudaStream_t st) {
     constexpr int kSub = 12, kSplit = 4;
     using Sh = Shape<kSub>;
-    auto fn = k_rows_phase_reduce_split<kSub, kSplit, CPLX, PADDED>;
+    auto fn = k_rows_phase_reduce_split<kSub, kSplit, CPLX, PAD>;
     const size_t smem = (size_t)(Sh::kTw + Sh::kArray + 256) * sizeof(float2) +
-                        (size_t)Sh::N * (sizeof(float2) + (CPLX ? 0 : 1) * sizeof(float));
+                        (size_t)Sh::T * Crop<PAD>::NJ * (sizeof(float2) + (CPLX ? 0 : 1) * sizeof(float));
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     fn<<<kSplit * P.Ni, Sh::T, smem, st>>>(P, grids, wsum, pix_turns, pix_scale, twid + Shape<14>::kTw,
@@ -1055,17 +1077,25 @@ template <int LOG2N>
 cudaError_t fused_n(const PhaseParams& P, const float2* grids, const double* wsum, const uint2* pix_turns,
                     const float* pix_scale, const float2* twid, float* image_real, float2* image_complex,
                     const Occupancy& occ, cudaStream_t st) {
-    const bool padded = P.Ni != P.N;
+    const int pad = P.Ni == P.N ? 0 : 2 * P.Ni == P.N ? 1 : 2;
+#define RICK_FUSED_PAD(fn_pad0, fn_pad1, fn_pad2) (pad == 0 ? fn_pad0 : pad == 1 ? fn_pad1 : fn_pad2)
 #define RICK_FUSED_ARGS P, grids, wsum, pix_turns, pix_scale, twid, image_real, image_complex, occ, st
     if constexpr (LOG2N == 14) {
         if (image_complex != nullptr)
-            return padded ? fused_split<true, true>(RICK_FUSED_ARGS) : fused_split<true, false>(RICK_FUSED_ARGS);
-        return padded ? fused_split<false, true>(RICK_FUSED_ARGS) : fused_split<false, false>(RICK_FUSED_ARGS);
+            return RICK_FUSED_PAD((fused_split<true, 0>(RICK_FUSED_ARGS)), (fused_split<true, 1>(RICK_FUSED_ARGS)),
+                                  (fused_split<true, 2>(RICK_FUSED_ARGS)));
+        return RICK_FUSED_PAD((fused_split<false, 0>(RICK_FUSED_ARGS)), (fused_split<false, 1>(RICK_FUSED_ARGS)),
+                              (fused_split<false, 2>(RICK_FUSED_ARGS)));
     } else {
         if (image_complex != nullptr)
-            return padded ? fused_one<LOG2N, true, true>(RICK_FUSED_ARGS) : fused_one<LOG2N, true, false>(RICK_FUSED_ARGS);
-        return padded ? fused_one<LOG2N, false, true>(RICK_FUSED_ARGS) : fused_one<LOG2N, false, false>(RICK_FUSED_ARGS);
+            return RICK_FUSED_PAD((fused_one<LOG2N, true, 0>(RICK_FUSED_ARGS)),
+                                  (fused_one<LOG2N, true, 1>(RICK_FUSED_ARGS)),
+                                  (fused_one<LOG2N, true, 2>(RICK_FUSED_ARGS)));
+        return RICK_FUSED_PAD((fused_one<LOG2N, false, 0>(RICK_FUSED_ARGS)),
+                              (fused_one<LOG2N, false, 1>(RICK_FUSED_ARGS)),
+                              (fused_one<LOG2N, false, 2>(RICK_FUSED_ARGS)));
     }
+#undef RICK_FUSED_PAD
 #undef RICK_FUSED_ARGS
 }
 

@@ -306,65 +306,16 @@ __device__ __forceinline__ void accumulate_range(const GridParams& G,
                 const float4 f = stg4[r];
                 const int ij = stg_ij[r];
                 const int i0 = (ij & 0xffff) - 256, j0 = (ij >> 16) - 256;
-                if constexpr (SS == 8 && !TABLE) {
-                    // a lane owns both words of cell (a, rl + 4 pp), pp = 0, 1:
-                    // rows step by 4, so its checkerboard sign and x tap are
-                    // fixed for the record; rows rl, rl + 1 are 16 banks apart
-                    const int a = lane & 7, rl = lane >> 3;
-                    const int i = i0 + a;
-                    const bool col_in = (unsigned)i < (unsigned)T;
+                const float wv = comp ? f.w : f.z;
+                const int n16 = (S * S + 15) & ~15;
+                for (int c = cl; c < n16; c += 16) {
+                    const int a = c % S, b = min(c / S, S - 1);
                     const float ga = __shfl_sync(kFull, tap, tb + a);
-                    const float sg = ((i + j0 + rl) & 1) ? -ga : ga;
-                    const float gre = sg * f.z, gim = sg * f.w;
-                    float2* cell = reinterpret_cast<float2*>(buf) + (j0 + rl) * P + i;
-#pragma unroll
-                    for (int pp = 0; pp < 2; ++pp) {
-                        const int b = rl + 4 * pp;
-                        const float gb = __shfl_sync(kFull, tap, tb + 8 + b);
-                        if (col_in && (unsigned)(j0 + b) < (unsigned)T) {
-                            float2* c = cell + 4 * P * pp;
-                            float2 v = *c;
-                            v.x = fmaf(gre, gb, v.x);
-                            v.y = fmaf(gim, gb, v.y);
-                            *c = v;
-                        }
-                    }
-                } else if constexpr (SS == 4 || SS == 8) {
-                    // a lane keeps column a and steps kRows (even) rows per pass,
-                    // so its checkerboard sign and x tap are fixed for the record
-                    constexpr int kRows = 16 / SS;
-                    const int a = cl % SS, rl = cl / SS;
-                    const int i = i0 + a;
-                    const bool col_in = (unsigned)i < (unsigned)T;
-                    const float wv = comp ? f.w : f.z;
-                    const float ga = __shfl_sync(kFull, tap, tb + a);
-                    const float sw = ((i + j0 + rl) & 1) ? -wv : wv;
-                    const float gw = sw * ga;
-                    float* cell = buf + 2 * ((j0 + rl) * P + i) + comp;
-#pragma unroll
-                    for (int pp = 0; pp < SS / kRows; ++pp) {
-                        const int b = rl + kRows * pp;
-                        const float gb = __shfl_sync(kFull, tap, tb + SS + b);
-                        if (col_in && (unsigned)(j0 + b) < (unsigned)T) {
-                            float* c = cell + 2 * kRows * P * pp;
-                            if (TABLE)
-                                *c = fmaf(sw, fmaf(ga, gb, stg_corr[r * 20 + 4 * b + a]), *c);
-                            else
-                                *c = fmaf(gw, gb, *c);
-                        }
-                    }
-                } else {
-                    const float wv = comp ? f.w : f.z;
-                    const int n16 = (S * S + 15) & ~15;
-                    for (int c = cl; c < n16; c += 16) {
-                        const int a = c % S, b = min(c / S, S - 1);
-                        const float ga = __shfl_sync(kFull, tap, tb + a);
-                        const float gb = __shfl_sync(kFull, tap, tb + S + b);
-                        const int i = i0 + a, j = j0 + c / S;
-                        if (c < S * S && (unsigned)i < (unsigned)T && (unsigned)j < (unsigned)T) {
-                            float* cell = buf + 2 * (j * P + i) + comp;
-                            *cell = fmaf(((i + j) & 1) ? -wv : wv, ga * gb, *cell);
-                        }
+                    const float gb = __shfl_sync(kFull, tap, tb + S + b);
+                    const int i = i0 + a, j = j0 + c / S;
+                    if (c < S * S && (unsigned)i < (unsigned)T && (unsigned)j < (unsigned)T) {
+                        float* cell = buf + 2 * (j * P + i) + comp;
+                        *cell = fmaf(((i + j) & 1) ? -wv : wv, ga * gb, *cell);
                     }
                 }
                 __syncwarp();
@@ -374,11 +325,150 @@ __device__ __forceinline__ void accumulate_range(const GridParams& G,
     }
 }
 
+// Supports 5 to 8 (separable kernels): what a record needs is prepared once by
+// one lane and read by the 32 that add it.  Lane r of a batch of 32 records
+// evaluates all 2S taps of record r -- the tap index is a compile-time constant,
+// so the coefficients are constant-bank operands -- multiplies the x taps by W V,
+// folds the checkerboard sign (-1)^(i+j) into both, and writes a slot of kSlot
+// floats: 8 products (re, im), then the y taps as the pairs (b, b + 4).  The
+// position, the columns and the rows of the footprint that lie inside the tile
+// travel in one word through a shuffle.  A lane then owns the cells (a, rl) and
+// (a, rl + 4) of every footprint: per record it makes three shared or shuffle
+// reads, two mask tests and two read-modify-writes.
+//
+// Against lanes that evaluate two records' taps at a time and fetch each by
+// shuffle (81 instructions per record and tile visited): 512 tiles of 60 records,
+// S = 7 (which took the general path, a division per cell), 203 -> 14 us; 16384^2,
+// S = 7, 11.7 M visibilities 6.5 -> 1.0 ms; 4096^2, S = 8, 30.6 M 3.95 -> 2.2 ms;
+// with a w-kernel, 15.3 M records, 1.98 -> 1.25 ms.  Now the load/store unit binds
+// it: some 12 shared-memory wavefronts a record.
+constexpr int kSlot = 28;       // 112 bytes: 16-byte stores of 8 lanes fall on distinct banks
+constexpr int kCellBias = 1024; // offset of a footprint's first cell, which may lie before the tile
+
+__device__ __forceinline__ float tap_uniform(const GridParams& G, int a, float t) {
+    float acc = G.coef[a][kPolyDegree];
+#pragma unroll
+    for (int k = kPolyDegree - 1; k >= 0; --k) acc = fmaf(acc, t, G.coef[a][k]);
+    return acc;
+}
+
+template <int SS>
+__device__ __forceinline__ void accumulate_slots(const GridParams& G, const VisRecord* __restrict__ records,
+                                                 const uint32_t (&rng)[8], uint32_t beg, uint32_t end, float* buf,
+                                                 float* slots) {
+    static_assert(SS >= 5 && SS <= 8, "support");
+    const int T = G.T;
+    constexpr float kInvFrac = 1.0f / 16777216.0f;
+    const int lane = threadIdx.x & 31;
+    const int P = tile_pitch(T, SS);
+    const uint32_t n0 = rng[1] - rng[0], n1 = rng[3] - rng[2], n2 = rng[5] - rng[4];
+    const int a = lane & 7, rl = lane >> 3;
+    // this lane's bits of a record's word: column a and row rl, or row rl + 4
+    const uint32_t need0 = (1u << a) | (256u << rl), need1 = (1u << a) | (4096u << rl);
+    float2* cell0 = reinterpret_cast<float2*>(buf) + rl * P + a - kCellBias;
+    float* mine = slots + lane * kSlot;
+    const float2* xs = reinterpret_cast<const float2*>(slots) + a;
+    const float2* ys = reinterpret_cast<const float2*>(slots + 16) + rl;
+    for (uint32_t base = beg; base < end; base += 32u) {
+        const uint32_t g = base + lane;
+        uint32_t word = 0u;
+        if (g < end) {
+            uint32_t src;
+            int dx = 0, dy = 0;
+            if (g < n0) {
+                src = rng[0] + g;
+            } else if (g < n0 + n1) {
+                src = rng[2] + (g - n0);
+                dx = -T;
+            } else if (g < n0 + n1 + n2) {
+                src = rng[4] + (g - n0 - n1);
+                dy = -T;
+            } else {
+                src = rng[6] + (g - n0 - n1 - n2);
+                dx = -T;
+                dy = -T;
+            }
+            VisRecord rec = records[src];
+            // RICK_DEBUG: the first footprint cell lies in the record's own tile
+            // (a corrupt record is dropped; the masks below keep every access
+            // inside the tile in any build)
+            if (!RICK_DCHECK((int)(rec.px >> kFracBits) < T && (int)(rec.py >> kFracBits) < T,
+                             kCheckRecordCell, G.status)) {
+                rec.wv_re = rec.wv_im = 0.f;
+                rec.px = rec.py = 0;
+            }
+            const int i0 = (int)(rec.px >> kFracBits) + dx, j0 = (int)(rec.py >> kFracBits) + dy;
+            // taps inside the tile: [max(0, -i0), min(S, T - i0)); none if the
+            // record does not reach it
+            auto inside = [&](int first) {
+                const int lo = first < 0 ? min(-first, SS) : 0, hi = min(SS, max(T - first, 0));
+                return ((1u << hi) - 1u) & ~((1u << lo) - 1u);
+            };
+            const uint32_t cols = inside(i0), rows = inside(j0);
+            word = cols != 0u && rows != 0u ? cols | (rows << 8) | ((uint32_t)(j0 * P + i0 + kCellBias) << 16) : 0u;
+            const float tx = fmaf(2.0f, (float)(rec.px & kFracMask) * kInvFrac, -1.0f);
+            const float ty = fmaf(2.0f, (float)(rec.py & kFracMask) * kInvFrac, -1.0f);
+            const float sg = ((i0 + j0) & 1) ? -1.f : 1.f;
+            const float re = sg * rec.wv_re, im = sg * rec.wv_im;
+            float x[16], y[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const float gx = t < SS ? tap_uniform(G, t, tx) : 0.f, gy = t < SS ? tap_uniform(G, t, ty) : 0.f;
+                x[2 * t] = (t & 1 ? -re : re) * gx;
+                x[2 * t + 1] = (t & 1 ? -im : im) * gx;
+                y[t] = t & 1 ? -gy : gy;
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                *reinterpret_cast<float4*>(mine + 4 * t) = make_float4(x[4 * t], x[4 * t + 1], x[4 * t + 2], x[4 * t + 3]);
+            *reinterpret_cast<float4*>(mine + 16) = make_float4(y[0], y[4], y[1], y[5]);
+            *reinterpret_cast<float4*>(mine + 20) = make_float4(y[2], y[6], y[3], y[7]);
+        }
+        __syncwarp();
+        const int cnt = (int)min(32u, end - base);
+        auto add = [&](uint32_t w, float2 x, float2 y) {
+            float2* c = cell0 + (w >> 16);
+            if ((w & need0) == need0) {
+                float2 v = *c;
+                v.x = fmaf(x.x, y.x, v.x);
+                v.y = fmaf(x.y, y.x, v.y);
+                *c = v;
+            }
+            if ((w & need1) == need1) {
+                float2 v = c[4 * P];
+                v.x = fmaf(x.x, y.y, v.x);
+                v.y = fmaf(x.y, y.y, v.y);
+                c[4 * P] = v;
+            }
+            __syncwarp();   // the next record's cells may be these
+        };
+        int r = 0;
+        for (; r + 4 <= cnt; r += 4) {
+            float2 x[4], y[4];
+            uint32_t w[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                w[q] = __shfl_sync(kFull, word, r + q);
+                x[q] = xs[(r + q) * (kSlot / 2)];
+                y[q] = ys[(r + q) * (kSlot / 2)];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) add(w[q], x[q], y[q]);
+        }
+        for (; r < cnt; ++r)
+            add(__shfl_sync(kFull, word, r), xs[r * (kSlot / 2)], ys[r * (kSlot / 2)]);
+    }
+}
+
 // Shared memory of a gridder CTA of nw warps (bytes): one zero row, one
 // T x P complex tile per warp, per-warp record staging and chunk bounds.
-__host__ __device__ inline size_t grid_smem_bytes(int T, int P, int nw, int grab_max, bool table) {
+__host__ __device__ constexpr bool uses_slots(int SS) { return SS >= 5 && SS <= 8; }
+// staging bytes of a warp's 32 records: slots, or (fractions, W V) and the cell
+__host__ __device__ constexpr int staging_bytes(int SS) { return 32 * (uses_slots(SS) ? kSlot * 4 : (int)(sizeof(float4) + sizeof(int))); }
+
+__host__ __device__ inline size_t grid_smem_bytes(int T, int P, int nw, int grab_max, bool table, int SS) {
     return sizeof(float) * (2 * (size_t)T + (size_t)nw * 2 * T * P) +
-           (size_t)nw * 32 * (sizeof(float4) + sizeof(int)) +
+           (size_t)nw * staging_bytes(SS) +
            sizeof(uint32_t) * (size_t)nw * 9 * grab_max +
            (table ? (size_t)nw * 32 * 20 * sizeof(float) : 0);
 }
@@ -409,10 +499,12 @@ __global__ void k_grid(GridParams G, const uint32_t* __restrict__ offsets,
     float2* zrow = reinterpret_cast<float2*>(smem);                 // T zero cells
     float* bufs = smem + 2 * T;
     float* buf = bufs + warp * tile_f;                              // this warp's tile
-    float4* stg4_all = reinterpret_cast<float4*>(bufs + nw * tile_f);
-    float4* stg4 = stg4_all + warp * 32;
-    int* stg_ij = reinterpret_cast<int*>(stg4_all + nw * 32) + warp * 32;
-    uint32_t* rng_all = reinterpret_cast<uint32_t*>(reinterpret_cast<int*>(stg4_all + nw * 32) + nw * 32) +
+    // staging: slots, or per warp 32 float4 and (after all of those) 32 ints
+    float* stg_all = bufs + nw * tile_f;
+    float* slots = stg_all + warp * 32 * kSlot;
+    float4* stg4 = reinterpret_cast<float4*>(stg_all) + warp * 32;
+    int* stg_ij = reinterpret_cast<int*>(reinterpret_cast<float4*>(stg_all) + nw * 32) + warp * 32;
+    uint32_t* rng_all = reinterpret_cast<uint32_t*>(stg_all + (size_t)nw * staging_bytes(SS) / 4) +
                         warp * 9 * kMaxWarpGrab;
     uint32_t* items = rng_all + 8 * kMaxWarpGrab;
     // learned-kernel staging; 16-byte aligned (the tiles, the zero row and
@@ -422,10 +514,17 @@ __global__ void k_grid(GridParams G, const uint32_t* __restrict__ offsets,
     float* stg_corr = TABLE ? tbl_base + warp * 32 * 20 : nullptr;
     const uint32_t tiles = (uint32_t)NT * NT;
     const uint32_t row_bytes = (uint32_t)T * sizeof(float2);
+    // records [beg, end) of a tile's range into this warp's tile
+    auto accumulate = [&](const uint32_t (&rng)[8], uint32_t beg, uint32_t end, int k, const float (&cf)[kPolyDegree + 1]) {
+        if constexpr (uses_slots(SS))
+            accumulate_slots<SS>(G, records, rng, beg, end, buf, slots);
+        else
+            accumulate_range<TABLE, SS>(G, records, rng, beg, end, k, buf, P, cf, stg4, stg_ij, stg_corr);
+    };
     // this lane's tap polynomial: lane (m, q) of a tap group of 2S lanes
     // evaluates tap q mod S (x taps q < S, y taps q >= S); zero beyond the groups
-    float cf[kPolyDegree + 1];
-    {
+    float cf[kPolyDegree + 1] = {};
+    if (!uses_slots(SS)) {
         const int S = SS > 0 ? SS : G.S;
         const int S2 = 2 * S, m = lane / S2, ta = (lane - m * S2) % S;
 #pragma unroll
@@ -484,7 +583,7 @@ __global__ void k_grid(GridParams G, const uint32_t* __restrict__ offsets,
         const int kk = (int)(plane % G.nk);
         const int ty = (int)(tile / NT), tx = (int)(tile - (uint32_t)ty * NT);
         float2* out = grids + ((uint64_t)plane * N + (uint64_t)ty * T) * N + (uint64_t)tx * T;
-        accumulate_range<TABLE, SS>(G, records, rng, beg, end, G.k0 + kk, buf, P, cf, stg4, stg_ij, stg_corr);
+        accumulate(rng, beg, end, G.k0 + kk, cf);
         __syncthreads();
         // sum the warps' tiles into warp 0's in warp order, clearing the others
         {
@@ -557,7 +656,7 @@ __global__ void k_grid(GridParams G, const uint32_t* __restrict__ offsets,
                 }
                 continue;
             }
-            accumulate_range<TABLE, SS>(G, records, rng, 0u, total, G.k0 + kk, buf, P, cf, stg4, stg_ij, stg_corr);
+            accumulate(rng, 0u, total, G.k0 + kk, cf);
             fence_async_shared();
             __syncwarp();
             for (int r = lane; r < T; r += 32)
@@ -594,7 +693,7 @@ cudaError_t launch_one(const GridParams& G, const uint32_t* offsets, const VisRe
                        cudaStream_t stream) {
     const int P = tile_pitch(G.T, SS > 0 ? SS : G.S);
     const int nw = threads / 32;
-    const size_t smem = grid_smem_bytes(G.T, P, nw, kMaxWarpGrab, TABLE);
+    const size_t smem = grid_smem_bytes(G.T, P, nw, kMaxWarpGrab, TABLE, SS);
     auto fn = k_grid<TABLE, SS>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -603,10 +702,14 @@ cudaError_t launch_one(const GridParams& G, const uint32_t* offsets, const VisRe
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     uint64_t blocks = (uint64_t)per_sm * num_sms;
-    const uint64_t need = (2ull * G.n_items + (uint64_t)G.grab * nw - 1) / ((uint64_t)G.grab * nw);
+    // fewer tiles than resident warps x grab: one tile a warp at a time, so that
+    // tiles run side by side (512 tiles of 60 records: 4 in turn took 4 times as long)
+    GridParams g = G;
+    while (g.grab > 1 && (uint64_t)g.n_items < blocks * nw * g.grab) g.grab >>= 1;
+    const uint64_t need = (2ull * g.n_items + (uint64_t)g.grab * nw - 1) / ((uint64_t)g.grab * nw);
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
-    fn<<<(unsigned)blocks, threads, smem, stream>>>(G, offsets, records, grids, counter);
+    fn<<<(unsigned)blocks, threads, smem, stream>>>(g, offsets, records, grids, counter);
     return cudaGetLastError();
 }
 
@@ -691,6 +794,8 @@ cudaError_t launch_grid(const GridParams& G, const uint32_t* offsets, const VisR
     } else {
         switch (G.S) {
             case 4: e = launch_one<false, 4>(G, offsets, records, grids, work_counter, threads, num_sms, stream); break;
+            case 5: e = launch_one<false, 5>(G, offsets, records, grids, work_counter, threads, num_sms, stream); break;
+            case 6: e = launch_one<false, 6>(G, offsets, records, grids, work_counter, threads, num_sms, stream); break;
             case 7: e = launch_one<false, 7>(G, offsets, records, grids, work_counter, threads, num_sms, stream); break;
             case 8: e = launch_one<false, 8>(G, offsets, records, grids, work_counter, threads, num_sms, stream); break;
             default: e = launch_one<false, 0>(G, offsets, records, grids, work_counter, threads, num_sms, stream); break;

@@ -21,16 +21,14 @@
 // stores each visibility once with its halo class.
 //
 // Records of the tile's own bins and of the three neighbour bins that spill
-// into it form one index range.  Each warp owns a band of tile rows and is
-// the only writer of its cells, so accumulation is plain FP32 load-add-store
-// in a fixed order (no shared-memory atomics, which for FP32 are
-// compare-and-swap loops, and a result that does not depend on scheduling).
-// A warp loads 32 records at once (one per lane), keeps those that reach its
-// band and walks them one by one: lanes 0..S-1 and 16..16+S-1 evaluate the 2S
-// one-dimensional taps (fitted polynomials), and the footprint cells inside
-// the band are covered 16 per instruction, an even/odd lane pair adding the
-// re/im parts of one cell.  The learned support-4 kernel adds a non-separable
-// correction interpolated from a per-plane lattice table.
+// into it form one index range.  A warp is the only writer of its tile buffer,
+// so accumulation is plain FP32 load-add-store in a fixed order (no
+// shared-memory atomics, which for FP32 are compare-and-swap loops, and a result
+// that does not depend on scheduling).  A warp takes 32 records at once, one per
+// lane, each lane prepares its record, and the warp adds them one by one
+// (accumulate_slots, accumulate_slots4; accumulate_range for other supports).
+// The learned support-4 kernel adds a non-separable correction interpolated from
+// a per-plane lattice table.
 #include <algorithm>
 #include <cmath>
 
@@ -54,28 +52,25 @@ __device__ __forceinline__ float tap_poly(const float (&cf)[kPolyDegree + 1], fl
     return acc;
 }
 
-// Learned correction taps c = 4b + a of one record: bilinear interpolation
-// of the plane's (L+1)^2 x 16 lattice table at (fx, fy), written to out[0..15].
-__device__ __forceinline__ void table_taps(const GridParams& G, int k, float fx, float fy,
-                                           float* out) {
-    const int L = G.lattice;
-    const float X = fx * L, Y = fy * L;
-    const int ix = min((int)X, L - 1), iy = min((int)Y, L - 1);
-    const float ax = X - ix, ay = Y - iy;
-    const size_t row = (size_t)(L + 1);
-    const float4* t00 = reinterpret_cast<const float4*>(G.table + (((size_t)k * row + iy) * row + ix) * 16);
-    const float4* t10 = t00 + 4;
-    const float4* t01 = t00 + row * 4;
-    const float4* t11 = t01 + 4;
-    const float w00 = (1.f - ax) * (1.f - ay), w10 = ax * (1.f - ay), w01 = (1.f - ax) * ay,
-                w11 = ax * ay;
+// Learned correction of a warp's 32 records: bilinear interpolation of the plane's
+// (L+1)^2 x 16 lattice table, four lanes a record and 16 bytes a lane, so that a
+// warp access takes eight 64-byte rows (a lane gathering its own record's rows took
+// 32 lines an access, three times the load/store cycles of adding the record).
+// Lane r passes record r's lattice row `at` and offsets; the 16 taps of record r go
+// to slots[r stride ..].
+__device__ __forceinline__ void table_taps(const GridParams& G, int at, float ax, float ay, float* slots, int stride) {
+    const int lane = threadIdx.x & 31, quad = lane & 3;
+    const size_t row = (size_t)(G.lattice + 1) * 4;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const float4 a = __ldg(t00 + q), b = __ldg(t10 + q), c = __ldg(t01 + q), d = __ldg(t11 + q);
-        out[4 * q + 0] = w00 * a.x + w10 * b.x + w01 * c.x + w11 * d.x;
-        out[4 * q + 1] = w00 * a.y + w10 * b.y + w01 * c.y + w11 * d.y;
-        out[4 * q + 2] = w00 * a.z + w10 * b.z + w01 * c.z + w11 * d.z;
-        out[4 * q + 3] = w00 * a.w + w10 * b.w + w01 * c.w + w11 * d.w;
+    for (int h = 0; h < 4; ++h) {
+        const int r = 8 * h + (lane >> 2);
+        const float x = __shfl_sync(kFull, ax, r), y = __shfl_sync(kFull, ay, r);
+        const float4* t = reinterpret_cast<const float4*>(G.table) + (size_t)__shfl_sync(kFull, at, r) * 4 + quad;
+        const float4 a = __ldg(t), b = __ldg(t + 4), c = __ldg(t + row), d = __ldg(t + row + 4);
+        const float w00 = (1.f - x) * (1.f - y), w10 = x * (1.f - y), w01 = (1.f - x) * y, w11 = x * y;
+        *reinterpret_cast<float4*>(slots + r * stride + 4 * quad) =
+            make_float4(w00 * a.x + w10 * b.x + w01 * c.x + w11 * d.x, w00 * a.y + w10 * b.y + w01 * c.y + w11 * d.y,
+                        w00 * a.z + w10 * b.z + w01 * c.z + w11 * d.z, w00 * a.w + w10 * b.w + w01 * c.w + w11 * d.w);
     }
 }
 
@@ -176,28 +171,70 @@ __global__ void k_schedule(GridParams G, const uint32_t* __restrict__ offsets,
 // rows 16 banks apart; S = 4: four rows 8 banks apart).
 __host__ __device__ constexpr int tile_pitch(int T, int S) { return S == 4 ? T + 4 : T + 8; }
 
-// Accumulate records [beg, end) of one tile's record range into buf
-// (interleaved re/im floats, row pitch P cells), by one warp that is the only
-// writer of buf: plain FP32 load-add-store in bin order, so no atomics and a
-// fixed order of additions.  rng: the tile's bin bounds -- own [0,1) all
-// classes, left [2,3), up [4,5), up-left [6,7); a neighbour's records are
-// relative to its origin (dx, dy = -T).  The warp stages 32 records at a time
-// in shared memory (fractions, W V, footprint start) and walks them: lanes
-// 0..S-1 / 16..16+S-1 evaluate the 2S 1-D taps, and the footprint is covered
-// 16 cells per instruction, an even/odd lane pair holding the re/im words of
-// one cell.
-template <bool TABLE, int SS>
-__device__ __forceinline__ void accumulate_range(const GridParams& G,
-                                                 const VisRecord* __restrict__ records,
-                                                 const uint32_t (&rng)[8], uint32_t beg,
-                                                 uint32_t end, int k, float* buf, int P,
-                                                 const float (&cf)[kPolyDegree + 1],
-                                                 float4* stg4, int* stg_ij, float* stg_corr) {
-    const int S = SS > 0 ? SS : G.S;
+// Record g of a tile's range (own bins, then the left, upper and upper-left
+// neighbours' spilling classes), its footprint starting at (i0, j0) of the tile.
+__device__ __forceinline__ VisRecord tile_record(const GridParams& G, const VisRecord* __restrict__ records,
+                                                 const uint32_t (&rng)[8], uint32_t g, int& i0, int& j0) {
+    const uint32_t n0 = rng[1] - rng[0], n1 = rng[3] - rng[2], n2 = rng[5] - rng[4];
     const int T = G.T;
+    uint32_t src;
+    int dx = 0, dy = 0;
+    if (g < n0) {
+        src = rng[0] + g;
+    } else if (g < n0 + n1) {
+        src = rng[2] + (g - n0);
+        dx = -T;
+    } else if (g < n0 + n1 + n2) {
+        src = rng[4] + (g - n0 - n1);
+        dy = -T;
+    } else {
+        src = rng[6] + (g - n0 - n1 - n2);
+        dx = -T;
+        dy = -T;
+    }
+    VisRecord rec = records[src];
+    // RICK_DEBUG: the first footprint cell lies in the record's own tile (a corrupt
+    // record is dropped; the masks and clips below keep every access inside the
+    // tile in any build)
+    if (!RICK_DCHECK((int)(rec.px >> kFracBits) < T && (int)(rec.py >> kFracBits) < T, kCheckRecordCell, G.status)) {
+        rec.wv_re = rec.wv_im = 0.f;
+        rec.px = rec.py = 0;
+    }
+    i0 = (int)(rec.px >> kFracBits) + dx;
+    j0 = (int)(rec.py >> kFracBits) + dy;
+    return rec;
+}
+
+constexpr int kCellBias = 1024; // offset of a footprint's first cell, which may lie before the tile
+
+// The columns (bits 0..7) and rows (8..15) of a footprint of support S starting at
+// (i0, j0) that lie inside the tile, and the offset of its first cell (biased, 16
+// bits); 0 if it does not reach the tile.
+template <int S>
+__device__ __forceinline__ uint32_t footprint_word(int T, int P, int i0, int j0) {
+    auto inside = [&](int first) {
+        const int lo = first < 0 ? min(-first, S) : 0, hi = min(S, max(T - first, 0));
+        return ((1u << hi) - 1u) & ~((1u << lo) - 1u);
+    };
+    const uint32_t cols = inside(i0), rows = inside(j0);
+    return cols != 0u && rows != 0u ? cols | (rows << 8) | ((uint32_t)(j0 * P + i0 + kCellBias) << 16) : 0u;
+}
+
+// The other supports (1 to 3, 9 to 16): accumulate records [beg, end) of one tile's
+// record range into buf (interleaved re/im floats, row pitch P cells), by one warp
+// that is the only writer of buf: plain FP32 load-add-store in bin order, so no
+// atomics and a fixed order of additions.  rng: the tile's bin bounds -- own [0,1)
+// all classes, left [2,3), up [4,5), up-left [6,7); a neighbour's records are
+// relative to its origin.  The warp stages 32 records at a time in shared memory
+// (fractions, W V, footprint start) and walks them: lanes 0..S-1 / S..2S-1 of a tap
+// group evaluate the 2S 1-D taps, and the footprint is covered 16 cells per
+// instruction, an even/odd lane pair holding the re/im words of one cell.
+__device__ __forceinline__ void accumulate_range(const GridParams& G, const VisRecord* __restrict__ records,
+                                                 const uint32_t (&rng)[8], uint32_t beg, uint32_t end, float* buf,
+                                                 int P, const float (&cf)[kPolyDegree + 1], float4* stg4, int* stg_ij) {
+    const int S = G.S, T = G.T;
     constexpr float kInvFrac = 1.0f / 16777216.0f;
     const int lane = threadIdx.x & 31;
-    const uint32_t n0 = rng[1] - rng[0], n1 = rng[3] - rng[2], n2 = rng[5] - rng[4];
     const int comp = lane & 1, cl = lane >> 1;       // cell slot 0..15 of a pass
     // tap groups: 32 / 2S records share one tap evaluation; lane (m, q)
     const int S2 = 2 * S, RG = 32 / S2;
@@ -205,46 +242,11 @@ __device__ __forceinline__ void accumulate_range(const GridParams& G,
     for (uint32_t base = beg; base < end; base += 32u) {
         const uint32_t g = base + lane;
         if (g < end) {
-            uint32_t src;
-            int dx = 0, dy = 0;
-            if (g < n0) {
-                src = rng[0] + g;
-            } else if (g < n0 + n1) {
-                src = rng[2] + (g - n0);
-                dx = -T;
-            } else if (g < n0 + n1 + n2) {
-                src = rng[4] + (g - n0 - n1);
-                dy = -T;
-            } else {
-                src = rng[6] + (g - n0 - n1 - n2);
-                dx = -T;
-                dy = -T;
-            }
-            VisRecord rec = records[src];
-            // RICK_DEBUG: the first footprint cell lies in the record's own tile
-            // (a corrupt record is dropped; the cell clipping below keeps every
-            // access inside the tile in any build)
-            if (!RICK_DCHECK((int)(rec.px >> kFracBits) < T && (int)(rec.py >> kFracBits) < T,
-                             kCheckRecordCell, G.status)) {
-                rec.wv_re = rec.wv_im = 0.f;
-                rec.px = rec.py = 0;
-            }
-            const int i0 = (int)(rec.px >> kFracBits) + dx, j0 = (int)(rec.py >> kFracBits) + dy;
+            int i0, j0;
+            const VisRecord rec = tile_record(G, records, rng, g, i0, j0);
             stg4[lane] = make_float4((float)(rec.px & kFracMask) * kInvFrac,
                                      (float)(rec.py & kFracMask) * kInvFrac, rec.wv_re, rec.wv_im);
             stg_ij[lane] = (i0 + 256) | ((j0 + 256) << 16);
-            if (TABLE) {
-                // the record's 16 correction taps, interpolated by its own lane:
-                // 16 independent 16-byte loads per lane, the 32 records of the
-                // batch in parallel (one round trip per batch); row stride 20
-                float corr[16];
-                table_taps(G, k, (float)(rec.px & kFracMask) * kInvFrac,
-                           (float)(rec.py & kFracMask) * kInvFrac, corr);
-#pragma unroll
-                for (int t = 0; t < 16; t += 4)
-                    *reinterpret_cast<float4*>(stg_corr + lane * 20 + t) =
-                        make_float4(corr[t], corr[t + 1], corr[t + 2], corr[t + 3]);
-            }
         }
         __syncwarp();
         const int cnt = (int)min(32u, end - base);
@@ -265,42 +267,6 @@ __device__ __forceinline__ void accumulate_range(const GridParams& G,
             const float tap = tap_next;
             if (r0 + RG < cnt) tap_next = group_taps(r0 + RG);
             const int nr = min(RG, cnt - r0);
-            if constexpr (SS == 4) {
-                // two records per pass, 16 lanes each (lane = cell 4b + a, both
-                // words), when their footprints do not overlap; else one by one
-                const int h = lane >> 4, c = lane & 15, a = c & 3, b = c >> 2;
-                for (int mm = 0; mm < nr; mm += 2) {
-                    const bool pair = mm + 1 < nr;
-                    const int ijA = stg_ij[r0 + mm], ijB = pair ? stg_ij[r0 + mm + 1] : ijA;
-                    const int dxi = (ijA & 0xffff) - (ijB & 0xffff), dyj = (ijA >> 16) - (ijB >> 16);
-                    const bool apart = pair && (dxi >= 4 || dxi <= -4 || dyj >= 4 || dyj <= -4);
-                    for (int step = 0; step < 2; ++step) {
-                        // step 0: record mm (half 0) and, if apart, mm + 1 (half 1);
-                        // step 1: record mm + 1 alone when the two overlap
-                        if (step == 1 && (!pair || apart)) break;
-                        const int mine = step == 0 ? mm + h : mm + 1;
-                        const bool act = step == 0 ? (h == 0 || apart) : h == 1;
-                        const int r = r0 + mine;
-                        const float4 f = stg4[min(r, cnt - 1)];
-                        const int ij = h == 0 ? (step == 0 ? ijA : ijB) : ijB;
-                        const int i0 = (ij & 0xffff) - 256, j0 = (ij >> 16) - 256;
-                        const float ga = __shfl_sync(kFull, tap, min(mine, RG - 1) * S2 + a);
-                        const float gb = __shfl_sync(kFull, tap, min(mine, RG - 1) * S2 + 4 + b);
-                        const int i = i0 + a, j = j0 + b;
-                        if (act && (unsigned)i < (unsigned)T && (unsigned)j < (unsigned)T) {
-                            float g = ga * gb;
-                            if (TABLE) g += stg_corr[r * 20 + c];
-                            if ((i + j) & 1) g = -g;
-                            float2* cp = reinterpret_cast<float2*>(buf) + j * P + i;
-                            float2 v = *cp;
-                            v.x = fmaf(f.z, g, v.x);
-                            v.y = fmaf(f.w, g, v.y);
-                            *cp = v;
-                        }
-                        __syncwarp();
-                    }
-                }
-            } else {
             for (int mm = 0; mm < nr; ++mm) {
                 const int r = r0 + mm, tb = mm * S2;
                 const float4 f = stg4[r];
@@ -320,12 +286,11 @@ __device__ __forceinline__ void accumulate_range(const GridParams& G,
                 }
                 __syncwarp();
             }
-            }
         }
     }
 }
 
-// Supports 5 to 8 (separable kernels): what a record needs is prepared once by
+// Supports 5 to 8 (separable kernels; 4 below): what a record needs is prepared once by
 // one lane and read by the 32 that add it.  Lane r of a batch of 32 records
 // evaluates all 2S taps of record r -- the tap index is a compile-time constant,
 // so the coefficients are constant-bank operands -- multiplies the x taps by W V,
@@ -343,7 +308,6 @@ __device__ __forceinline__ void accumulate_range(const GridParams& G,
 // with a w-kernel, 15.3 M records, 1.98 -> 1.25 ms.  Now the load/store unit binds
 // it: some 12 shared-memory wavefronts a record.
 constexpr int kSlot = 28;       // 112 bytes: 16-byte stores of 8 lanes fall on distinct banks
-constexpr int kCellBias = 1024; // offset of a footprint's first cell, which may lie before the tile
 
 __device__ __forceinline__ float tap_uniform(const GridParams& G, int a, float t) {
     float acc = G.coef[a][kPolyDegree];
@@ -361,7 +325,6 @@ __device__ __forceinline__ void accumulate_slots(const GridParams& G, const VisR
     constexpr float kInvFrac = 1.0f / 16777216.0f;
     const int lane = threadIdx.x & 31;
     const int P = tile_pitch(T, SS);
-    const uint32_t n0 = rng[1] - rng[0], n1 = rng[3] - rng[2], n2 = rng[5] - rng[4];
     const int a = lane & 7, rl = lane >> 3;
     // this lane's bits of a record's word: column a and row rl, or row rl + 4
     const uint32_t need0 = (1u << a) | (256u << rl), need1 = (1u << a) | (4096u << rl);
@@ -373,39 +336,9 @@ __device__ __forceinline__ void accumulate_slots(const GridParams& G, const VisR
         const uint32_t g = base + lane;
         uint32_t word = 0u;
         if (g < end) {
-            uint32_t src;
-            int dx = 0, dy = 0;
-            if (g < n0) {
-                src = rng[0] + g;
-            } else if (g < n0 + n1) {
-                src = rng[2] + (g - n0);
-                dx = -T;
-            } else if (g < n0 + n1 + n2) {
-                src = rng[4] + (g - n0 - n1);
-                dy = -T;
-            } else {
-                src = rng[6] + (g - n0 - n1 - n2);
-                dx = -T;
-                dy = -T;
-            }
-            VisRecord rec = records[src];
-            // RICK_DEBUG: the first footprint cell lies in the record's own tile
-            // (a corrupt record is dropped; the masks below keep every access
-            // inside the tile in any build)
-            if (!RICK_DCHECK((int)(rec.px >> kFracBits) < T && (int)(rec.py >> kFracBits) < T,
-                             kCheckRecordCell, G.status)) {
-                rec.wv_re = rec.wv_im = 0.f;
-                rec.px = rec.py = 0;
-            }
-            const int i0 = (int)(rec.px >> kFracBits) + dx, j0 = (int)(rec.py >> kFracBits) + dy;
-            // taps inside the tile: [max(0, -i0), min(S, T - i0)); none if the
-            // record does not reach it
-            auto inside = [&](int first) {
-                const int lo = first < 0 ? min(-first, SS) : 0, hi = min(SS, max(T - first, 0));
-                return ((1u << hi) - 1u) & ~((1u << lo) - 1u);
-            };
-            const uint32_t cols = inside(i0), rows = inside(j0);
-            word = cols != 0u && rows != 0u ? cols | (rows << 8) | ((uint32_t)(j0 * P + i0 + kCellBias) << 16) : 0u;
+            int i0, j0;
+            const VisRecord rec = tile_record(G, records, rng, g, i0, j0);
+            word = footprint_word<SS>(T, P, i0, j0);
             const float tx = fmaf(2.0f, (float)(rec.px & kFracMask) * kInvFrac, -1.0f);
             const float ty = fmaf(2.0f, (float)(rec.py & kFracMask) * kInvFrac, -1.0f);
             const float sg = ((i0 + j0) & 1) ? -1.f : 1.f;
@@ -460,17 +393,110 @@ __device__ __forceinline__ void accumulate_slots(const GridParams& G, const VisR
     }
 }
 
+// Support 4, separable or with the learned correction: the same split, with the 16
+// signed taps of a record (the separable ones plus the learned correction) and
+// its W V in the slot; lane (c, comp) owns one word of cell c = 4b + a, so all 32
+// lanes work on every record.  2 M visibilities on 16 planes of 2048^2 (GB300, whole
+// planes written): learned 315 -> 194 us, separable 198 -> 157 us.
+constexpr int kSlot4 = 20;      // 80 bytes: 16-byte stores of 8 lanes fall on distinct banks
+
+template <bool TABLE>
+__device__ __forceinline__ void accumulate_slots4(const GridParams& G, const VisRecord* __restrict__ records,
+                                                  const uint32_t (&rng)[8], uint32_t beg, uint32_t end, int k,
+                                                  float* buf, float* slots) {
+    const int T = G.T;
+    constexpr float kInvFrac = 1.0f / 16777216.0f;
+    const int lane = threadIdx.x & 31;
+    const int P = tile_pitch(T, 4);
+    const int c = lane >> 1, comp = lane & 1, a = c & 3, b = c >> 2;
+    const uint32_t need = (1u << a) | (256u << b);
+    float* cell0 = buf + 2 * (b * P + a - kCellBias) + comp;
+    float* mine = slots + lane * kSlot4;
+    for (uint32_t base = beg; base < end; base += 32u) {
+        const uint32_t g = base + lane;
+        uint32_t word = 0u;
+        VisRecord rec = {};
+        int i0 = 0, j0 = 0;
+        if (g < end) rec = tile_record(G, records, rng, g, i0, j0);
+        const float fx = (float)(rec.px & kFracMask) * kInvFrac, fy = (float)(rec.py & kFracMask) * kInvFrac;
+        if (TABLE) {
+            const int L = G.lattice;
+            const float X = fx * L, Y = fy * L;
+            const int ix = min((int)X, L - 1), iy = min((int)Y, L - 1);
+            table_taps(G, (k * (L + 1) + iy) * (L + 1) + ix, X - ix, Y - iy, slots, kSlot4);
+            __syncwarp();
+        }
+        if (g < end) {
+            word = footprint_word<4>(T, P, i0, j0);
+            const float tx = fmaf(2.0f, fx, -1.0f), ty = fmaf(2.0f, fy, -1.0f);
+            float tap[16];
+            if (TABLE) {
+#pragma unroll
+                for (int t = 0; t < 16; t += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(mine + t);
+                    tap[t] = v.x;
+                    tap[t + 1] = v.y;
+                    tap[t + 2] = v.z;
+                    tap[t + 3] = v.w;
+                }
+            }
+            float gx[4], gy[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                gx[t] = tap_uniform(G, t, tx);
+                gy[t] = tap_uniform(G, t, ty);
+            }
+            const bool odd = ((i0 + j0) & 1) != 0;
+#pragma unroll
+            for (int t = 0; t < 16; ++t) {
+                float v = gx[t & 3] * gy[t >> 2];
+                if (TABLE) v += tap[t];
+                tap[t] = ((t ^ (t >> 2)) & 1 ? !odd : odd) ? -v : v;
+            }
+#pragma unroll
+            for (int t = 0; t < 16; t += 4)
+                *reinterpret_cast<float4*>(mine + t) = make_float4(tap[t], tap[t + 1], tap[t + 2], tap[t + 3]);
+            *reinterpret_cast<float2*>(mine + 16) = make_float2(rec.wv_re, rec.wv_im);
+        }
+        __syncwarp();
+        const int cnt = (int)min(32u, end - base);
+        auto add = [&](uint32_t w, float t, float wv) {
+            if ((w & need) == need) {
+                float* at = cell0 + 2 * (w >> 16);
+                *at = fmaf(wv, t, *at);
+            }
+            __syncwarp();   // the next record's cells may be these
+        };
+        int r = 0;
+        for (; r + 4 <= cnt; r += 4) {
+            float t[4], wv[4];
+            uint32_t w[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                w[q] = __shfl_sync(kFull, word, r + q);
+                t[q] = slots[(r + q) * kSlot4 + c];
+                wv[q] = slots[(r + q) * kSlot4 + 16 + comp];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) add(w[q], t[q], wv[q]);
+        }
+        for (; r < cnt; ++r)
+            add(__shfl_sync(kFull, word, r), slots[r * kSlot4 + c], slots[r * kSlot4 + 16 + comp]);
+    }
+}
+
 // Shared memory of a gridder CTA of nw warps (bytes): one zero row, one
 // T x P complex tile per warp, per-warp record staging and chunk bounds.
-__host__ __device__ constexpr bool uses_slots(int SS) { return SS >= 5 && SS <= 8; }
+__host__ __device__ constexpr bool uses_slots(int SS) { return SS >= 4 && SS <= 8; }
 // staging bytes of a warp's 32 records: slots, or (fractions, W V) and the cell
-__host__ __device__ constexpr int staging_bytes(int SS) { return 32 * (uses_slots(SS) ? kSlot * 4 : (int)(sizeof(float4) + sizeof(int))); }
+__host__ __device__ constexpr int staging_bytes(int SS) { 
+    return 32 * (SS == 4 ? kSlot4 * 4 : uses_slots(SS) ? kSlot * 4 : (int)(sizeof(float4) + sizeof(int)));
+}
 
-__host__ __device__ inline size_t grid_smem_bytes(int T, int P, int nw, int grab_max, bool table, int SS) {
+__host__ __device__ inline size_t grid_smem_bytes(int T, int P, int nw, int grab_max, int SS) {
     return sizeof(float) * (2 * (size_t)T + (size_t)nw * 2 * T * P) +
            (size_t)nw * staging_bytes(SS) +
-           sizeof(uint32_t) * (size_t)nw * 9 * grab_max +
-           (table ? (size_t)nw * 32 * 20 * sizeof(float) : 0);
+           sizeof(uint32_t) * (size_t)nw * 9 * grab_max;
 }
 
 // The gridder.  work_counter: [0] dense-tile queue, [1..3] list lengths,
@@ -501,25 +527,22 @@ __global__ void k_grid(GridParams G, const uint32_t* __restrict__ offsets,
     float* buf = bufs + warp * tile_f;                              // this warp's tile
     // staging: slots, or per warp 32 float4 and (after all of those) 32 ints
     float* stg_all = bufs + nw * tile_f;
-    float* slots = stg_all + warp * 32 * kSlot;
+    float* slots = stg_all + warp * (staging_bytes(SS) / 4);
     float4* stg4 = reinterpret_cast<float4*>(stg_all) + warp * 32;
     int* stg_ij = reinterpret_cast<int*>(reinterpret_cast<float4*>(stg_all) + nw * 32) + warp * 32;
     uint32_t* rng_all = reinterpret_cast<uint32_t*>(stg_all + (size_t)nw * staging_bytes(SS) / 4) +
                         warp * 9 * kMaxWarpGrab;
     uint32_t* items = rng_all + 8 * kMaxWarpGrab;
-    // learned-kernel staging; 16-byte aligned (the tiles, the zero row and
-    // the 928 bytes per warp of record staging and chunk bounds before it are
-    // all multiples of 16 bytes), so rows of 20 floats take float4 stores
-    float* tbl_base = reinterpret_cast<float*>(rng_all - warp * 9 * kMaxWarpGrab + nw * 9 * kMaxWarpGrab);
-    float* stg_corr = TABLE ? tbl_base + warp * 32 * 20 : nullptr;
     const uint32_t tiles = (uint32_t)NT * NT;
     const uint32_t row_bytes = (uint32_t)T * sizeof(float2);
     // records [beg, end) of a tile's range into this warp's tile
     auto accumulate = [&](const uint32_t (&rng)[8], uint32_t beg, uint32_t end, int k, const float (&cf)[kPolyDegree + 1]) {
-        if constexpr (uses_slots(SS))
+        if constexpr (SS == 4)
+            accumulate_slots4<TABLE>(G, records, rng, beg, end, k, buf, slots);
+        else if constexpr (uses_slots(SS))
             accumulate_slots<SS>(G, records, rng, beg, end, buf, slots);
         else
-            accumulate_range<TABLE, SS>(G, records, rng, beg, end, k, buf, P, cf, stg4, stg_ij, stg_corr);
+            accumulate_range(G, records, rng, beg, end, buf, P, cf, stg4, stg_ij);
     };
     // this lane's tap polynomial: lane (m, q) of a tap group of 2S lanes
     // evaluates tap q mod S (x taps q < S, y taps q >= S); zero beyond the groups
@@ -693,7 +716,7 @@ cudaError_t launch_one(const GridParams& G, const uint32_t* offsets, const VisRe
                        cudaStream_t stream) {
     const int P = tile_pitch(G.T, SS > 0 ? SS : G.S);
     const int nw = threads / 32;
-    const size_t smem = grid_smem_bytes(G.T, P, nw, kMaxWarpGrab, TABLE, SS);
+    const size_t smem = grid_smem_bytes(G.T, P, nw, kMaxWarpGrab, SS);
     auto fn = k_grid<TABLE, SS>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -257,7 +257,6 @@ k_place(PlaceParams P, const double* __restrict__ uvw, const double* __restrict_
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int c = (int)(tid0 % P.C);
     const double sc = chan_scale[c];
-    s_wsum[threadIdx.x] = 0.0;
     if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0ull;
     __syncthreads();
 
@@ -317,9 +316,17 @@ k_place(PlaceParams P, const double* __restrict__ uvw, const double* __restrict_
         }
     }
 
-    // per-channel weight sums: block reduction in shared memory, then global
-    if (P.C <= kPlaceThreads) {
-        if (my_wsum != 0.0) atomicAdd(&s_wsum[c], my_wsum);
+    // per-channel weight sums, without FP64 shared-memory atomics (compare-and-swap
+    // loops: with one channel the 256 threads of a block took turns on one address,
+    // most of the 22 us of a 20 k visibility call): lanes of one channel are added by
+    // shuffles where the channels repeat within a warp, then one thread per channel
+    // adds the warps' (or the threads') sums in order
+    const bool in_warp = P.C <= 32 && (P.C & (P.C - 1)) == 0;
+    if (in_warp) {
+        for (int o = 16; o >= P.C; o >>= 1) my_wsum += __shfl_xor_sync(0xffffffffu, my_wsum, o);
+        if (lane < P.C) s_wsum[(threadIdx.x >> 5) * P.C + lane] = my_wsum;
+    } else if (P.C <= kPlaceThreads) {
+        s_wsum[threadIdx.x] = my_wsum;
     } else if (my_wsum != 0.0) {
         atomicAdd(&weight_sum[c], my_wsum);
     }
@@ -330,8 +337,13 @@ k_place(PlaceParams P, const double* __restrict__ uvw, const double* __restrict_
         if (d) atomicAdd(&s_cnt[1], (unsigned long long)d);
     }
     __syncthreads();
-    if (P.C <= kPlaceThreads && threadIdx.x < P.C && s_wsum[threadIdx.x] != 0.0)
-        atomicAdd(&weight_sum[threadIdx.x], s_wsum[threadIdx.x]);
+    if (P.C <= kPlaceThreads && threadIdx.x < P.C) {
+        // thread t < C of the block has channel c, and so has every C-th entry
+        const int n = in_warp ? kPlaceThreads / 32 * P.C : kPlaceThreads;
+        double w = 0.0;
+        for (int t = threadIdx.x; t < n; t += P.C) w += s_wsum[t];
+        if (w != 0.0) atomicAdd(&weight_sum[c], w);
+    }
     if (threadIdx.x < 2 && s_cnt[threadIdx.x]) atomicAdd(&counts[threadIdx.x], s_cnt[threadIdx.x]);
 }
 

@@ -881,8 +881,8 @@ rick_status phase_impl(rick_plan* P, const float* grids, int c0, int c1, int k0,
     int launches = 0;
     rick_status s = check_launch(
         launch_phase_reduce(pp, reinterpret_cast<const float2*>(grids), weight_sum + c0,
-                            P->d_inv_taper, image_real, reinterpret_cast<float2*>(image_complex),
-                            st, &launches),
+                            P->d_inv_taper, P->d_pix_turns, P->d_pix_scale, image_real,
+                            reinterpret_cast<float2*>(image_complex), st, &launches),
         "phase kernel");
     P->launches += launches;
     return s;

@@ -229,9 +229,10 @@ cudaError_t launch_grid(const GridParams& G, const uint32_t* offsets, const VisR
                         float2* grids, uint32_t* work_counter, int threads, int num_sms,
                         cudaStream_t stream, int* launches);
 
+// pix_turns, pix_scale: the plan's per-pixel table (launch_pixel_phase), or null
 cudaError_t launch_phase_reduce(const PhaseParams& P, const float2* grids, const double* wsum,
-                                const float* taper, float* image_real, float2* image_complex,
-                                cudaStream_t stream, int* launches);
+                                const float* taper, const uint2* pix_turns, const float* pix_scale,
+                                float* image_real, float2* image_complex, cudaStream_t stream, int* launches);
 
 // prediction (degridding)
 cudaError_t launch_model_planes(const PhaseParams& P, const float* image, const float* inv_taper,

@@ -1088,8 +1088,12 @@ rick_status degrid_impl(rick_plan* P, const float* grids, int c0, int c1, int k0
     G.w_support = c.w_support >= 2 ? c.w_support : 0;
     G.status = P->d_status;
     std::memcpy(G.coef, P->tap_coef, sizeof G.coef);
+    // the work list takes the binning's unsorted records' place (free once binned):
+    // 16 bytes a record, two entries
+    G.entries = reinterpret_cast<uint2*>(P->d_stage);
+    G.entry_cap = (uint32_t)std::min<int64_t>(2 * P->cap_vis, 0xFFFFFFFFll);
     P->last_stream = st;
-    RK_CUDA(cudaMemsetAsync(P->d_counter, 0, sizeof(uint32_t), st));
+    RK_CUDA(cudaMemsetAsync(P->d_counter, 0, 2 * sizeof(uint32_t), st));
     int launches = 0;
     rick_status s = check_launch(
         launch_degrid(G, P->d_offsets, P->d_records, reinterpret_cast<const float2*>(grids),

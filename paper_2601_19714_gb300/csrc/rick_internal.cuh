@@ -114,6 +114,8 @@ struct GridParams {
     // only, never the unreached tiles.  light_cap >= the launch's tiles.
     uint32_t* light;
     uint32_t light_cap;
+    uint2* entries;       // prediction: the work list, (tile, first record) (rick_degrid.cu)
+    uint32_t entry_cap;
     int w_support;        // prediction: >= 2 accumulates the Sw partial predictions
     // 1: tiles that no record reaches are not written (the zero fill is left
     // out); the planes are then only valid where tile_reach() > 0
@@ -241,7 +243,8 @@ cudaError_t launch_model_planes(const PhaseParams& P, const float* image, const 
 // Gathers the prediction of every record binned for prediction whose
 // (channel, plane) lies in G's range from the transformed planes `grids`
 // (layout as for the gridder) into vis_out[index] (conjugated where flagged).
-// work_counter: 1 word, zero on entry.
+// work_counter: 2 words, zero on entry; G.entries holds entry_cap >= 2 entries
+// per binned record.
 cudaError_t launch_degrid(const GridParams& G, const uint32_t* offsets, const VisRecord* records,
                           const float2* grids, float2* vis_out, uint32_t* work_counter, int threads,
                           int num_sms, cudaStream_t stream, int* launches);

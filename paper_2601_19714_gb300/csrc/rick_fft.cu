@@ -816,21 +816,15 @@ k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __rest
     const size_t NN = (size_t)N * N, NNi = (size_t)Ni * Ni;
     const bool warp_mask = occ.tshift >= 5 && T >= 32;
     const int lane = b & 31;
-    // the tile columns of plane r that the column pass reads
-    auto live_cols = [&](int r) -> uint32_t {
-        uint32_t live = 0xffffu;
-        if (occ.col != nullptr) {
-            const uint8_t* cm = occ.col + (size_t)r * occ.NT;
-            if (warp_mask) {
-                const bool on = lane < 16 && __ldg(cm + (((b & ~31) + T * lane) >> occ.tshift)) != 0;
-                live = __ballot_sync(0xffffffffu, on);
-            } else {
-                live = 0;
+    // the tile columns of plane r that the column pass reads: the mask bytes, loaded
+    // before the transform, and the 16 bits, needed after it
+    auto load_mask = [&](int r) -> uint32_t {
+        if (occ.col == nullptr) return 0xffffu;
+        const uint8_t* cm = occ.col + (size_t)r * occ.NT;
+        if (warp_mask) return lane < 16 ? __ldg(cm + (((b & ~31) + T * lane) >> occ.tshift)) : 0u;
+        uint32_t live = 0;
 #pragma unroll
-                for (int t2 = 0; t2 < 16; ++t2)
-                    live |= (__ldg(cm + ((b + T * t2) >> occ.tshift)) != 0 ? 1u : 0u) << t2;
-            }
-        }
+        for (int t2 = 0; t2 < 16; ++t2) live |= (__ldg(cm + ((b + T * t2) >> occ.tshift)) != 0 ? 1u : 0u) << t2;
         return live;
     };
     const uint2* turns = pix_turns + (size_t)qi * Ni;
@@ -891,8 +885,9 @@ k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __rest
                 ph[t2] = make_float2(fmaf(ph[t2].x, z.x, -ph[t2].y * z.y), fmaf(ph[t2].x, z.y, ph[t2].y * z.x));
             }
             kcur = kk + 1;
+            const uint32_t mask = load_mask(r);
             transform<LOG2N, false>(a, buf, b, tw, x);
-            const uint32_t live = live_cols(r);
+            const uint32_t live = occ.col != nullptr && warp_mask ? __ballot_sync(0xffffffffu, mask != 0u) : mask;
             float2* row = grids + (size_t)r * NN + (size_t)q * N;
 #pragma unroll
             for (int j = 0; j < 16; ++j)

@@ -126,7 +126,8 @@ __device__ __forceinline__ uint32_t tile_bound(const GridParams& G, const uint32
 // Scheduling pass: the record count of every tile, and the tiles with at
 // least 64T, 16T, 4T records appended to the three lists (warp-aggregated
 // atomics on the list lengths counts[0..2]); with G.light, every other tile
-// with a record to the light list (length counts[4]).
+// with a record to the light list (length counts[4]); with G.huge, the chunks of the
+// tiles to split (number counts[5]).
 __global__ void k_schedule(GridParams G, const uint32_t* __restrict__ offsets,
                            uint32_t* __restrict__ counts) {
     const int lane = threadIdx.x & 31;
@@ -142,6 +143,14 @@ __global__ void k_schedule(GridParams G, const uint32_t* __restrict__ offsets,
             for (int q = 0; q < 8; ++q) b[q] = tile_bound(G, offsets, item, q);
             const uint32_t R = (b[1] - b[0]) + (b[3] - b[2]) + (b[5] - b[4]) + (b[7] - b[6]);
             level = R >= th1 ? 0 : R >= th2 ? 1 : R >= th3 ? 2 : R > 0 ? 3 : 4;
+            if (G.huge != nullptr && R >= 2u * huge_chunk(G.T)) {
+                const uint32_t n = min((R + huge_chunk(G.T) - 1u) / huge_chunk(G.T), kHugeChunks);
+                const uint32_t at = atomicAdd(&counts[5], n);
+                if (at <= G.huge_cap && n <= G.huge_cap - at) {
+                    G.huge_done[at] = 0u;
+                    for (uint32_t q = 0; q < n; ++q) G.huge[at + q] = make_uint4(item, q, n, at);
+                }
+            }
         }
 #pragma unroll
         for (int lv = 0; lv < 4; ++lv) {
@@ -500,9 +509,11 @@ __host__ __device__ inline size_t grid_smem_bytes(int T, int P, int nw, int grab
 }
 
 // The gridder.  work_counter: [0] dense-tile queue, [1..3] list lengths,
-// [4] tile queue.
-//  Phase 1 -- dense tiles (the first two longest-first lists, >= 16T
-//  records), one per CTA: the tile's records are split evenly over the warps,
+// [4] tile queue, [5] light list length, [6] chunks of split tiles.
+//  Phase 1 -- first the chunks of the tiles with thousands of records (an array's core
+//  on a small mesh: one CTA a tile made a serial chain of 28 ms out of 6 M
+//  visibilities on 512^2), whose partial tiles the last CTA of a tile adds up; then
+//  dense tiles (the first two longest-first lists, >= 16T records), one per CTA: the tile's records are split evenly over the warps,
 //  each accumulates its share into its own tile buffer, the buffers are summed
 //  in warp order (a fixed order), and the CTA hands the rows to the bulk-copy
 //  engine.
@@ -564,7 +575,7 @@ __global__ void k_grid(GridParams G, const uint32_t* __restrict__ offsets,
     // longest-first lists (if any): their lengths, capped; an overflow (which
     // the capacity bound excludes) falls back to natural order for all tiles
     uint32_t n1 = 0, n2 = 0, n3 = 0, th3 = 0xffffffffu;
-    uint32_t n_light = 0;
+    uint32_t n_light = 0, n_huge = 0;
     bool light = false;   // phase 2 visits the lists only (sparse mode)
     if (G.lists) {
         n1 = __ldg(work_counter + 1);
@@ -574,6 +585,10 @@ __global__ void k_grid(GridParams G, const uint32_t* __restrict__ offsets,
             n1 = n2 = n3 = 0;
         } else {
             th3 = 4u * T;
+            if (G.huge != nullptr) {
+                n_huge = __ldg(work_counter + 6);
+                if (n_huge > G.huge_cap) n_huge = 0;
+            }
             if (G.light != nullptr && G.skip_empty) {
                 n_light = __ldg(work_counter + 5);
                 light = n_light <= G.light_cap;
@@ -587,9 +602,13 @@ __global__ void k_grid(GridParams G, const uint32_t* __restrict__ offsets,
     for (;;) {
         if (threadIdx.x == 0) s_heavy = atomicAdd(work_counter, 1u);
         __syncthreads();
-        const uint32_t h = s_heavy;
-        if (h >= nH) break;
-        const uint32_t item = h < n1 ? G.lists[h] : G.lists[G.list_cap + (h - n1)];
+        const uint32_t hh = s_heavy;
+        if (hh >= n_huge + nH) break;
+        // the chunks of the split tiles first, then the dense tiles
+        const uint32_t h = hh - n_huge;
+        uint4 part = make_uint4(0u, 0u, 1u, 0u);
+        if (hh < n_huge) part = G.huge[hh];
+        const uint32_t item = hh < n_huge ? part.x : h < n1 ? G.lists[h] : G.lists[G.list_cap + (h - n1)];
         if (!RICK_DCHECK(item < G.n_items, kCheckGridItem, G.status)) {   // uniform over the CTA
             __syncthreads();   // everyone has read s_heavy before thread 0 rewrites it
             continue;
@@ -600,8 +619,13 @@ __global__ void k_grid(GridParams G, const uint32_t* __restrict__ offsets,
 #pragma unroll
         for (int q = 0; q < 8; ++q) rng[q] = s_hrng[q];
         const uint32_t R = (rng[1] - rng[0]) + (rng[3] - rng[2]) + (rng[5] - rng[4]) + (rng[7] - rng[6]);
-        const uint32_t beg = (uint32_t)((uint64_t)R * warp / nw);
-        const uint32_t end = (uint32_t)((uint64_t)R * (warp + 1) / nw);
+        if (hh >= n_huge && n_huge != 0u && R >= 2u * huge_chunk(T)) {   // split (uniform over the CTA)
+            __syncthreads();   // s_heavy and s_hrng have been read
+            continue;
+        }
+        const uint32_t share = part.y * nw + warp, shares = part.z * nw;
+        const uint32_t beg = (uint32_t)((uint64_t)R * share / shares);
+        const uint32_t end = (uint32_t)((uint64_t)R * (share + 1) / shares);
         const uint32_t plane = item / tiles, tile = item - plane * tiles;
         const int kk = (int)(plane % G.nk);
         const int ty = (int)(tile / NT), tx = (int)(tile - (uint32_t)ty * NT);
@@ -623,6 +647,38 @@ __global__ void k_grid(GridParams G, const uint32_t* __restrict__ offsets,
                     *tw = make_float4(0.f, 0.f, 0.f, 0.f);
                 }
                 t0[e] = acc;
+            }
+        }
+        if (part.z > 1u) {
+            // a chunk of a split tile: its partial tile to memory; the CTA that
+            // finishes the tile's last chunk adds the partial tiles in chunk order
+            __syncthreads();
+            const int cells2 = T * T / 2, half = T / 2;   // cells two by two
+            float4* mine = G.huge_part + (size_t)(part.w + part.y) * cells2;
+            for (int e = threadIdx.x; e < cells2; e += blockDim.x) {
+                float4* c = reinterpret_cast<float4*>(bufs + 2 * ((e / half) * P + 2 * (e % half)));
+                mine[e] = *c;
+                *c = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            __threadfence();
+            __syncthreads();
+            if (threadIdx.x == 0) s_heavy = atomicAdd(G.huge_done + part.w, 1u) + 1u;
+            __syncthreads();
+            const bool last = s_heavy == part.z;
+            __syncthreads();   // s_heavy has been read
+            if (!last) continue;
+            __threadfence();
+            for (int e = threadIdx.x; e < cells2; e += blockDim.x) {
+                const float4* from = G.huge_part + (size_t)part.w * cells2 + e;
+                float4 acc = __ldcg(from);
+                for (uint32_t q = 1; q < part.z; ++q) {
+                    const float4 v = __ldcg(from + (size_t)q * cells2);
+                    acc.x += v.x;
+                    acc.y += v.y;
+                    acc.z += v.z;
+                    acc.w += v.w;
+                }
+                *reinterpret_cast<float4*>(bufs + 2 * ((e / half) * P + 2 * (e % half))) = acc;
             }
         }
         fence_async_shared();

@@ -108,6 +108,14 @@ struct GridParams {
     // first, then every other tile in natural order.  nullptr: natural order.
     uint32_t* lists;
     uint32_t list_cap;
+    // Optional, with lists: tiles of at least 2 huge_chunk(T) records, split over several
+    // CTAs.  work_counter[6] entries (tile, chunk, chunks, the tile's first entry),
+    // huge_cap at most (more: no tile is split), each with a T x T partial tile in
+    // huge_part and, at a tile's first entry, its finished chunks in huge_done.
+    uint4* huge;
+    uint32_t* huge_done;
+    float4* huge_part;
+    uint32_t huge_cap;
     // Sparse mode (skip_empty) only, optional: every other reached tile (fewer
     // than 4T records, at least one), listed by the scheduling pass
     // (work_counter[5] holds the count); the gridder then visits the lists
@@ -149,6 +157,15 @@ __device__ __forceinline__ uint32_t tile_reach(const uint32_t* __restrict__ offs
 inline uint32_t schedule_list_cap(int64_t max_vis, int T) {
     return (uint32_t)(max_vis / T + 64);
 }
+
+// Records of one CTA's share of a split tile at least (half the threshold): four
+// warps add 4096 in about 30 us, so one dense tile no longer outlasts the launch, and
+// its partial tile costs as much to write and read back as a few hundred records.
+__host__ __device__ constexpr uint32_t huge_chunk(int T) { return T > 32 ? 16384u : 4096u; }
+constexpr uint32_t kHugeChunks = 128;   // chunks a tile at most (the last CTA adds them up)
+inline uint32_t huge_list_cap(int64_t max_vis, int T) { return (uint32_t)(2 * max_vis / huge_chunk(T) + 64); }
+// bytes of the split tiles' memory: entries, counters, partial tiles
+inline size_t huge_bytes(uint32_t cap, int T) { return (size_t)cap * (sizeof(uint4) + 16 + sizeof(float2) * T * T); }
 
 // Fit the tap polynomials of a Gaussian or Kaiser-Bessel kernel of support S
 // (param = sigma or beta) into G.coef; returns the largest deviation from the

@@ -266,6 +266,89 @@ k_fft_rows(float2* __restrict__ grids, const float2* __restrict__ twid) {
     for (int j = 0; j < 16; ++j) __stcs(row + b + T * j, x[j]);
 }
 
+// The row transform of the fused passes: T threads of V values each, thread b from
+// inputs b + T t2 to outputs b + T j.  first() runs stage 0 and stores; after a
+// barrier rest() runs the others; after free() the buffer may be rewritten.
+//
+// The radix-16 transform above, except N = 256 (radix 4) and the model pass of N = 512
+// (radix 8): 64 threads a row, each value's chain a quarter or half as long, for a row
+// of a small mesh is latency only (16 threads of 16 values took 2.6 us a plane: rows of
+// 8 planes of 256^2 21.5 -> 13.6 us, model rows of 9 planes of 512^2 28.7 -> 22.5 us) --
+// exchanging through two buffers in turn, one barrier an exchange, with all N twiddles
+// W_N^k in the table.  Dense rows (k_fft_rows) are bound by HBM and stay at radix 16
+// (64-thread rows: 128 planes of 512^2 98 -> 110 us at best), and so does the imaging
+// pass of N = 512, which equals the separate calls to the last rounding.
+template <int LOG2N, bool INV>
+struct RowDft {
+    using Sh = Shape<LOG2N>;
+    static constexpr int V = 16, T = Sh::T, kBuf = Sh::kArray, kTable = Sh::kTw, kTableAt = 0;
+    static __device__ __forceinline__ void first(float2 (&a)[V], float2* buf, int b, const float2* tw) {
+        radix16_out<LOG2N, INV>(a, b, 0, buf, tw);
+    }
+    static __device__ __forceinline__ void rest(float2* buf, int b, const float2* tw, float2 (&x)[V]) {
+        middle_stages<LOG2N, INV>(buf, b, tw);
+        last_stage<LOG2N, INV>(buf, b, x);
+    }
+    static __device__ __forceinline__ void free() { __syncthreads(); }
+};
+
+template <int LOG2N, int RADIX, bool INV>
+struct RowDftSmall {
+    using Sh = Shape<LOG2N>;
+    static constexpr int N = Sh::N, V = RADIX, T = N / V, kBuf = 2 * N, kTable = N;
+    // after the stage tables, the 256 phasors and the column pass's tables
+    static constexpr int kTableAt = Sh::kTw + 256 + 16 * Sh::T + (Sh::kTw - 4 * Sh::T);
+    static constexpr int kLogV = V == 4 ? 2 : 3, kStages = LOG2N / kLogV;
+    static_assert(kStages * kLogV == LOG2N && kStages % 2 == (V == 4 ? 0 : 1), "stages");
+    template <int S>
+    static __device__ __forceinline__ void store(float2 (&a)[V], float2* buf, int b, const float2* tw) {
+        Dft<V, INV>::run(a);
+        constexpr int M = 1 << (kLogV * S);
+        const int t1 = b >> (kLogV * S), g = b & (M - 1);
+        float2* out = buf + t1 * V * M + g;
+        out[0] = a[0];
+#pragma unroll
+        for (int f = 1; f < V; ++f) {
+            float2 w = tw[t1 * f * M];
+            if (!INV) w.y = -w.y;
+            out[f * M] = cmulf(a[f], w);
+        }
+    }
+    template <int S>
+    static __device__ __forceinline__ void stages(float2* buf, int b, const float2* tw, float2 (&x)[V]) {
+        // stage S reads the half of the buffer that stage S - 1 wrote
+        const float2* in = buf + ((S - 1) & 1) * N;
+        float2 a[V];
+#pragma unroll
+        for (int t2 = 0; t2 < V; ++t2) a[t2] = in[b + T * t2];
+        if constexpr (S == kStages - 1) {
+            Dft<V, INV>::run(a);
+#pragma unroll
+            for (int j = 0; j < V; ++j) x[j] = a[j];
+        } else {
+            store<S>(a, buf + (S & 1) * N, b, tw);
+            __syncthreads();
+            stages<S + 1>(buf, b, tw, x);
+        }
+    }
+    static __device__ __forceinline__ void first(float2 (&a)[V], float2* buf, int b, const float2* tw) {
+        store<0>(a, buf, b, tw);
+    }
+    static __device__ __forceinline__ void rest(float2* buf, int b, const float2* tw, float2 (&x)[V]) {
+        stages<1>(buf, b, tw, x);
+    }
+    // kStages - 1 exchanges alternate between the halves.  An odd number of them (N =
+    // 256: three) ends on half 0, which the next row's stage 0 rewrites; an even one
+    // (N = 512: two) ends on half 1, whose readers the next row's first barrier holds
+    static __device__ __forceinline__ void free() {
+        if (kStages % 2 == 0) __syncthreads();
+    }
+};
+template <bool INV>
+struct RowDft<8, INV> : RowDftSmall<8, 4, INV> {};
+template <>
+struct RowDft<9, false> : RowDftSmall<9, 8, false> {};
+
 __device__ __forceinline__ uint32_t turns_q32(double t) {
     const double f = t - floor(t);  // [0, 1)
     return (uint32_t)__double2ull_rz(f * 4294967296.0);
@@ -333,38 +416,39 @@ __global__ void k_pixel_phase(PhaseParams P, const float* __restrict__ inv_taper
 // CTAs an SM that the fused row passes are compiled for: 16 warps, i.e. at most
 // 128 registers a thread (with the two CTAs of N = 4096 asked for at every
 // length, N = 2048 took 172 registers and ran 8 warps an SM: with the crop 264 ->
-// 122 us on 4 channels x 8 planes of a 2048^2 mesh; N = 256's 16 threads take a
-// whole warp's registers, so 16 CTAs are as many as 128 registers allow)
-constexpr int row_min_ctas(int log2n) { return log2n >= 13 ? 1 : log2n >= 9 ? (1 << (13 - log2n)) : 16; }
+// 122 us on 4 channels x 8 planes of a 2048^2 mesh)
+constexpr int row_min_ctas(int threads) { return threads >= 512 ? 1 : 512 / threads; }
 constexpr int kHornerBlock = 8;   // planes per Horner block of the fused row pass
 
-// The mesh pixels b + T j, j < 16, of a thread that a row pass keeps: all (PAD =
-// 0), the middle eight of a mesh twice the image (PAD = 1: exactly the image's),
-// or the middle four (PAD = 2: every padding by 4 or more, whose image pixels
+// The mesh pixels b + T j, j < V (16), of a thread that a row pass keeps: all (PAD =
+// 0), the middle half of a mesh twice the image (PAD = 1: exactly the image's),
+// or the middle quarter (PAD = 2: every padding by 4 or more, whose image pixels
 // among them are told apart at run time).  Phasing, summing and then dropping the
 // other pixels took a quarter of the pass: rows of a 4096^2 mesh padded by 2
 // (16 channels x 16 planes) 4.37 -> 3.60 ms, of an 8192^2 one (6 x 20) 14.4 ->
 // 11.9 ms.
-template <int PAD>
+template <int PAD, int V = 16>
 struct Crop {
-    static constexpr int J0 = PAD == 0 ? 0 : PAD == 1 ? 4 : 6;
-    static constexpr int NJ = PAD == 0 ? 16 : PAD == 1 ? 8 : 4;
+    static constexpr int J0 = PAD == 0 ? 0 : PAD == 1 ? V / 4 : V == 4 ? 1 : 3 * V / 8;
+    static constexpr int NJ = PAD == 0 ? V : PAD == 1 ? V / 2 : V == 4 ? 2 : V / 4;
     static constexpr bool kExact = PAD < 2;
 };
 
 template <int LOG2N, bool COMPLEX_OUT, int PAD>
-__global__ void __launch_bounds__((1 << LOG2N) / 16, row_min_ctas(LOG2N))
+__global__ void __launch_bounds__(RowDft<LOG2N, true>::T, row_min_ctas(RowDft<LOG2N, true>::T))
 k_rows_phase_reduce(PhaseParams P, const float2* __restrict__ grids, const double* __restrict__ wsum,
                     const uint2* __restrict__ pix_turns, const float* __restrict__ pix_scale,
                     const float2* __restrict__ twid, float* __restrict__ image_real,
                     float2* __restrict__ image_complex, Occupancy occ) {
     using Sh = Shape<LOG2N>;
-    using Cr = Crop<PAD>;
-    constexpr int N = Sh::N, T = Sh::T, J0 = Cr::J0, NJ = Cr::NJ;
+    using Rt = RowDft<LOG2N, true>;
+    constexpr int N = Sh::N, T = Rt::T, V = Rt::V;
+    using Cr = Crop<PAD, V>;
+    constexpr int J0 = Cr::J0, NJ = Cr::NJ;
     extern __shared__ __align__(16) float2 fsm[];
     float2* tw = fsm;
-    float2* buf = fsm + Sh::kTw;
-    float2* turn256 = buf + Sh::kArray;                          // e^(2 pi i j / 256)
+    float2* buf = fsm + Rt::kTable;
+    float2* turn256 = buf + Rt::kBuf;                          // e^(2 pi i j / 256)
     float2* zrot = turn256 + 256;                                // z = e^(-2 pi i dt) per pixel
     // the channel's finished blocks per pixel: Re of the phased sums
     float* part = reinterpret_cast<float*>(zrot + NJ * T);
@@ -375,7 +459,7 @@ k_rows_phase_reduce(PhaseParams P, const float2* __restrict__ grids, const doubl
     const int b = threadIdx.x, q = blockIdx.x;
     const float* scl = pix_scale + (size_t)q * Ni;               // per-pixel scale (read once per channel)
     const uint2* turns = pix_turns + (size_t)q * Ni;
-    load_tables<LOG2N>(twid, tw, b, T);
+    for (int j = b; j < Rt::kTable; j += T) tw[j] = __ldg(twid + Rt::kTableAt + j);
     for (int j = b; j < 256; j += T) turn256[j] = __ldg(twid + Sh::kTw + j);
 #pragma unroll 4
     for (int j = 0; j < NJ; ++j) {
@@ -397,33 +481,33 @@ k_rows_phase_reduce(PhaseParams P, const float2* __restrict__ grids, const doubl
     };
     // row q of plane r: the inputs b + T t2 of this thread; the unreached tile
     // columns are zero (the column pass did not touch them): not read
-    // With tiles of at least 32 columns (and N/16 >= 32) the tile column of
-    // input b + T t2 is the same for a whole warp: lanes 0..15 read the 16
-    // mask bytes and a ballot hands every lane the 16 bits.
+    // With tiles of at least 32 columns (and T >= 32) the tile column of input
+    // b + T t2 is the same for a whole warp: lanes 0..V-1 read the V mask bytes and
+    // a ballot hands every lane the bits.
     const bool warp_mask = occ.tshift >= 5 && T >= 32;
-    auto load_row = [&](int r, float2 (&v)[16]) {
+    auto load_row = [&](int r, float2 (&v)[V]) {
         const float2* row = grids + (size_t)r * NN + (size_t)(q + off) * N;
         if (occ.col != nullptr) {
             const uint8_t* cm = occ.col + (size_t)r * occ.NT;
             uint32_t live = 0;
             if (warp_mask) {
                 const int lane = b & 31;
-                const bool on = lane < 16 && __ldg(cm + (((b & ~31) + T * lane) >> occ.tshift)) != 0;
+                const bool on = lane < V && __ldg(cm + (((b & ~31) + T * lane) >> occ.tshift)) != 0;
                 live = __ballot_sync(0xffffffffu, on);
             } else {
 #pragma unroll
-                for (int t2 = 0; t2 < 16; ++t2)
+                for (int t2 = 0; t2 < V; ++t2)
                     live |= (__ldg(cm + ((b + T * t2) >> occ.tshift)) != 0 ? 1u : 0u) << t2;
             }
 #pragma unroll
-            for (int t2 = 0; t2 < 16; ++t2)
+            for (int t2 = 0; t2 < V; ++t2)
                 v[t2] = (live >> t2) & 1u ? __ldcs(row + b + T * t2) : make_float2(0.f, 0.f);
         } else {
 #pragma unroll
-            for (int t2 = 0; t2 < 16; ++t2) v[t2] = __ldcs(row + b + T * t2);
+            for (int t2 = 0; t2 < V; ++t2) v[t2] = __ldcs(row + b + T * t2);
         }
     };
-    float2 a[16], x[16];
+    float2 a[V], x[V];
     int r = next_row(0);
     if (r < n_rows) load_row(r, a);
     __syncthreads();
@@ -439,14 +523,13 @@ k_rows_phase_reduce(PhaseParams P, const float2* __restrict__ grids, const doubl
                     acc[j] = make_float2(fmaf(acc[j].x, z.x, -acc[j].y * z.y), fmaf(acc[j].x, z.y, acc[j].y * z.x));
                 }
             } else {
-                radix16_out<LOG2N, true>(a, b, 0, buf, tw);
+                Rt::first(a, buf, b, tw);
                 const int rn = next_row(r + 1);
                 if (rn < n_rows) load_row(rn, a);
                 r = rn;
                 __syncthreads();
-                middle_stages<LOG2N, true>(buf, b, tw);
-                last_stage<LOG2N, true>(buf, b, x);
-                __syncthreads();   // buf is rewritten by the next row's first stage
+                Rt::rest(buf, b, tw, x);
+                Rt::free();   // buf is rewritten by the next row's first stage
 #pragma unroll
                 for (int j = 0; j < NJ; ++j) {
                     const float2 z = zrot[b + T * j];
@@ -796,16 +879,17 @@ k_rows_phase_reduce_split(PhaseParams P, const float2* __restrict__ grids, const
 // reached tile columns are written (the column pass reads nothing else, and
 // the degridder only the reached tiles).
 template <int LOG2N>
-__global__ void __launch_bounds__((1 << LOG2N) / 16, row_min_ctas(LOG2N))
+__global__ void __launch_bounds__(RowDft<LOG2N, false>::T, row_min_ctas(RowDft<LOG2N, false>::T))
 k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __restrict__ pix_turns,
              const float* __restrict__ pix_model_scale, const float2* __restrict__ twid,
              float2* __restrict__ grids, Occupancy occ) {
     using Sh = Shape<LOG2N>;
-    constexpr int N = Sh::N, T = Sh::T;
+    using Rt = RowDft<LOG2N, false>;
+    constexpr int N = Sh::N, T = Rt::T, V = Rt::V;
     extern __shared__ __align__(16) float2 fsm[];
     float2* tw = fsm;
-    float2* buf = fsm + Sh::kTw;
-    float2* zrot = buf + Sh::kArray;                            // z = e^(-2 pi i dt) per pixel
+    float2* buf = fsm + Rt::kTable;
+    float2* zrot = buf + Rt::kBuf;                            // z = e^(-2 pi i dt) per pixel
     float* js = reinterpret_cast<float*>(zrot + N);             // J_c(p) times the pixel's scale
     // image row qi (blockIdx.x) is mesh row qi + off and mesh pixel pm image
     // pixel pm - off (a padded mesh holds the image in its central Ni x Ni;
@@ -821,16 +905,16 @@ k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __rest
     auto load_mask = [&](int r) -> uint32_t {
         if (occ.col == nullptr) return 0xffffu;
         const uint8_t* cm = occ.col + (size_t)r * occ.NT;
-        if (warp_mask) return lane < 16 ? __ldg(cm + (((b & ~31) + T * lane) >> occ.tshift)) : 0u;
+        if (warp_mask) return lane < V ? __ldg(cm + (((b & ~31) + T * lane) >> occ.tshift)) : 0u;
         uint32_t live = 0;
 #pragma unroll
-        for (int t2 = 0; t2 < 16; ++t2) live |= (__ldg(cm + ((b + T * t2) >> occ.tshift)) != 0 ? 1u : 0u) << t2;
+        for (int t2 = 0; t2 < V; ++t2) live |= (__ldg(cm + ((b + T * t2) >> occ.tshift)) != 0 ? 1u : 0u) << t2;
         return live;
     };
     const uint2* turns = pix_turns + (size_t)qi * Ni;
-    load_tables<LOG2N>(twid, tw, b, T);
+    for (int j = b; j < Rt::kTable; j += T) tw[j] = __ldg(twid + Rt::kTableAt + j);
 #pragma unroll 4
-    for (int t2 = 0; t2 < 16; ++t2) {
+    for (int t2 = 0; t2 < V; ++t2) {
         const int pm = b + T * t2, p = pm - off;
         float s = 0.f, c = 1.f;
         if ((unsigned)p < (unsigned)Ni)
@@ -842,7 +926,7 @@ k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __rest
         const float* ms = pix_model_scale + (size_t)qi * Ni;
         __syncthreads();   // the previous channel's js reads are done
 #pragma unroll 4
-        for (int t2 = 0; t2 < 16; ++t2) {
+        for (int t2 = 0; t2 < V; ++t2) {
             const int pm = b + T * t2, p = pm - off;
             js[pm] = (unsigned)p < (unsigned)Ni ? __ldg(jr + p) * __ldg(ms + p) : 0.f;
         }
@@ -850,7 +934,7 @@ k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __rest
         // plane of each block of kHornerBlock planes and advanced plane by plane
         // -- across skipped planes too, so that pruning does not change the
         // arithmetic
-        float2 ph[16];
+        float2 ph[V];
         int kcur = 0, block = -1;
         for (int kk = 0; kk < P.nk; ++kk) {
             const int r = cc * P.nk + kk;
@@ -860,7 +944,7 @@ k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __rest
                 kcur = block * kHornerBlock;
                 const uint32_t k = (uint32_t)(P.k_first + kcur);
 #pragma unroll
-                for (int t2 = 0; t2 < 16; ++t2) {
+                for (int t2 = 0; t2 < V; ++t2) {
                     const int p = b + T * t2 - off;
                     const uint2 t = (unsigned)p < (unsigned)Ni ? __ldg(&turns[p]) : make_uint2(0u, 0u);
                     float sn, cs;
@@ -870,14 +954,14 @@ k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __rest
             }
             for (; kcur < kk; ++kcur) {   // over skipped planes
 #pragma unroll
-                for (int t2 = 0; t2 < 16; ++t2) {
+                for (int t2 = 0; t2 < V; ++t2) {
                     const float2 z = zrot[b + T * t2];
                     ph[t2] = make_float2(fmaf(ph[t2].x, z.x, -ph[t2].y * z.y), fmaf(ph[t2].x, z.y, ph[t2].y * z.x));
                 }
             }
-            float2 a[16], x[16];
+            float2 a[V], x[V];
 #pragma unroll
-            for (int t2 = 0; t2 < 16; ++t2) {
+            for (int t2 = 0; t2 < V; ++t2) {
                 const int p = b + T * t2;
                 const float j = js[p];
                 const float2 z = zrot[p];
@@ -886,13 +970,15 @@ k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __rest
             }
             kcur = kk + 1;
             const uint32_t mask = load_mask(r);
-            transform<LOG2N, false>(a, buf, b, tw, x);
+            Rt::first(a, buf, b, tw);
+            __syncthreads();
+            Rt::rest(buf, b, tw, x);
             const uint32_t live = occ.col != nullptr && warp_mask ? __ballot_sync(0xffffffffu, mask != 0u) : mask;
             float2* row = grids + (size_t)r * NN + (size_t)q * N;
 #pragma unroll
-            for (int j = 0; j < 16; ++j)
+            for (int j = 0; j < V; ++j)
                 if ((live >> j) & 1u) __stcs(row + b + T * j, x[j]);
-            __syncthreads();   // buf is rewritten by the next plane's first stage
+            Rt::free();   // buf is rewritten by the next plane's first stage
         }
     }
 }
@@ -1042,11 +1128,12 @@ cudaError_t fused_one(const PhaseParams& P, const float2* grids, const double* w
     auto fn = k_rows_phase_reduce<LOG2N, CPLX, PAD>;
     // tables, the transform array and the 256 phasors, then per pixel z and
     // (real output) the partial sum
-    const size_t smem = (size_t)(Sh::kTw + Sh::kArray + 256) * sizeof(float2) +
-                        (size_t)Sh::T * Crop<PAD>::NJ * (sizeof(float2) + (CPLX ? 0 : 1) * sizeof(float));
+    using Rt = RowDft<LOG2N, true>;
+    const size_t smem = (size_t)(Rt::kTable + Rt::kBuf + 256) * sizeof(float2) +
+                        (size_t)Rt::T * Crop<PAD, Rt::V>::NJ * (sizeof(float2) + (CPLX ? 0 : 1) * sizeof(float));
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    fn<<<P.Ni, Sh::T, smem, st>>>(P, grids, wsum, pix_turns, pix_scale, twid, image_real, image_complex, occ);
+    fn<<<P.Ni, Rt::T, smem, st>>>(P, grids, wsum, pix_turns, pix_scale, twid, image_real, image_complex, occ);
     return cudaGetLastError();
 }
 
@@ -1156,7 +1243,7 @@ void append_pair_tables(int N, std::vector<float2>& out) {
 
 void fft_twiddles(int N, std::vector<float2>& out) {
     // N < 16384: the stage tables, then e^(2 pi i j / 256), j < 256, then the
-    // column pass's tables (append_pair_tables).
+    // column pass's tables (append_pair_tables) and, up to N = 512, all W_N^k.
     // N = 16384: the 4096-point tables of the split fused row pass follow,
     // then its split twiddles [r T + b] = e^(+2 pi i r b / N), r < 4, b < T = 256,
     // then e^(2 pi i j / 256), j < 256, then the four-step column pass's tables
@@ -1170,6 +1257,12 @@ void fft_twiddles(int N, std::vector<float2>& out) {
             out.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
         }
         append_pair_tables(N, out);
+        // N = 256, 512: every W_N^k, k < N, of the small row transforms
+        if (N <= 512)
+            for (int k = 0; k < N; ++k) {
+                const double a = 6.283185307179586476925 * (double)k / N;
+                out.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
+            }
     }
     if (log2_exact(N) == 14) {
         append_twiddles(4096, out);
@@ -1282,10 +1375,11 @@ cudaError_t launch_model_rows(const PhaseParams& P, const float* image, const ui
     case LG: {                                                                                      \
         using Sh = Shape<LG>;                                                                       \
         auto fn = k_model_rows<LG>;                                                                 \
-        const size_t smem = (size_t)(Sh::kTw + Sh::kArray + Sh::N) * sizeof(float2) + (size_t)Sh::N * sizeof(float); \
+        using Rt = RowDft<LG, false>;                                                               \
+        const size_t smem = (size_t)(Rt::kTable + Rt::kBuf + Sh::N) * sizeof(float2) + (size_t)Sh::N * sizeof(float); \
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);      \
         if (e == cudaSuccess) {                                                                     \
-            fn<<<P.Ni, Sh::T, smem, st>>>(P, image, pix_turns, pix_model_scale, twid, grids, occ); \
+            fn<<<P.Ni, Rt::T, smem, st>>>(P, image, pix_turns, pix_model_scale, twid, grids, occ); \
             e = cudaGetLastError();                                                                 \
         }                                                                                           \
         break;                                                                                      \

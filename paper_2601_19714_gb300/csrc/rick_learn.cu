@@ -27,11 +27,17 @@
 // i p/N), whose powers are the probe's constants (rounded from FP64 on the host).
 // A thread of the forward pass owns one probe and walks visibilities staged in
 // shared memory, so its sums stay in registers; a thread of the backward pass owns
-// one visibility and walks the probes.  Measured on GB300 (N = 2048, 2 M
+// one visibility and walks the probes.  I - D is a small difference of I and D, so the
+// loss magnifies the rounding of the two sums: a thread's FP32 sums cover one staged
+// block (32 terms) and go on in FP64 from there to the loss.  RMS relative error of the
+// loss against 64 bits over 6 to 8 seeds, at 2 M / 200 k / 20 k visibilities: FP32 sums
+// throughout 4.6e-6 / 1.5e-5 / 7.1e-6 (a warp reduction per pair 1.2e-5 / 1.7e-5 /
+// 2.2e-6), now 1.9e-6 / 2.7e-6 / 7.6e-7.  Measured on GB300 (N = 2048, 2 M
 // visibilities, 64 probes, lattice 32) against one visibility a thread in the
 // forward pass with a warp reduction per pair, 64-bit remainders and four phasors:
 // forward 3.37 -> 0.65 ms, backward 2.19 -> 0.39 ms, prediction of a field's sources
-// 0.6 -> 0.1 ms, a training step of four fields 25.2 -> 4.7 ms.
+// 0.6 -> 0.1 ms (each with FP32 sums throughout); a training step of four fields
+// 25.2 -> 4.96 ms, 4.75 of it before the FP64 sums.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -231,10 +237,10 @@ constexpr int kFwdRow = 6;     // float4 of a staged visibility: 16 taps, (W V, 
 __global__ void __launch_bounds__(256)
 k_learn_forward(const LearnVis* __restrict__ vis, const float2* __restrict__ wv,
                 const float* __restrict__ table, LearnConst C, KbTaps K, const Probe* __restrict__ probes,
-                const float2* __restrict__ ph, float* __restrict__ out) {
+                const float2* __restrict__ ph, double* __restrict__ out) {
     extern __shared__ __align__(16) float4 s_vis[];   // kFwdVis rows, then the phasors e^(2 pi i w_k delta_P)
     float2* s_ph = reinterpret_cast<float2*>(s_vis + kFwdVis * kFwdRow);
-    __shared__ float2 s_acc[4][kMaxProbes];
+    __shared__ double2 s_acc[4][kMaxProbes];
     const int tid = threadIdx.x, warp = tid >> 5;
     const int P = (warp & 1) * 32 + (tid & 31), quarter = warp >> 1;
     for (int i = tid; i < C.Nw * kMaxProbes; i += 256) s_ph[i] = ph[i];
@@ -242,7 +248,7 @@ k_learn_forward(const LearnVis* __restrict__ vis, const float2* __restrict__ wv,
     if (P < C.np) pr = probes[P];
     const bool idle = (warp & 1) * 32 >= C.np;
     const float inv_half_n = 2.0f / (float)C.N;
-    float img = 0.f, dft = 0.f;
+    double img64 = 0.0, dft64 = 0.0;
     for (int base = blockIdx.x * kFwdVis; base < C.nvis; base += gridDim.x * kFwdVis) {
         __syncthreads();   // the previous visibilities have been read (and the phasors are there)
         if (tid < kFwdVis) {
@@ -266,6 +272,7 @@ k_learn_forward(const LearnVis* __restrict__ vis, const float2* __restrict__ wv,
         __syncthreads();
         if (idle) continue;
         const float4* row = s_vis + quarter * (kFwdVis / 4) * kFwdRow;
+        float img = 0.f, dft = 0.f;
 #pragma unroll 2
         for (int r = 0; r < kFwdVis / 4; ++r, row += kFwdRow) {
             const float4 a = row[4], b = row[5];
@@ -290,33 +297,40 @@ k_learn_forward(const LearnVis* __restrict__ vis, const float2* __restrict__ wv,
             const float2 d = turn_phasor(fmaf(a.z, pr.pn, fmaf(a.w, pr.qn, fmaf(b.x, pr.delta, pr.turn))));
             dft = fmaf(c.x, d.x, fmaf(-c.y, d.y, dft));
         }
+        img64 += img;
+        dft64 += dft;
     }
-    s_acc[quarter][P] = make_float2(img, dft);
+    s_acc[quarter][P] = make_double2(img64, dft64);
     __syncthreads();
     if (tid < C.np) {
-        float2 t = s_acc[0][tid];
+        double2 t = s_acc[0][tid];
 #pragma unroll
         for (int q = 1; q < 4; ++q) {
             t.x += s_acc[q][tid].x;
             t.y += s_acc[q][tid].y;
         }
         const Probe& o = probes[tid];
-        atomicAdd(&out[2 * tid], o.scale_img * t.x * C.inv_wsum);
-        atomicAdd(&out[2 * tid + 1], o.scale_dft * t.y * C.inv_wsum);
+        atomicAdd(&out[2 * tid], (double)o.scale_img * t.x * (double)C.inv_wsum);
+        atomicAdd(&out[2 * tid + 1], (double)o.scale_dft * t.y * (double)C.inv_wsum);
     }
 }
 
 // loss = sum (I - D)^2 / sum D^2; ge[P] = dloss/dI_P (scaled by 1/sum W, which
-// the backward kernel's per-visibility terms omit).  One warp, two probes a lane.
-__global__ void k_learn_loss(const float* __restrict__ idft, int np, float inv_wsum,
-                             float* __restrict__ loss, float* __restrict__ ge) {
+// the backward kernel's per-visibility terms omit); idft[2P], idft[2P + 1] = I_P, D_P
+// rounded.  One warp, two probes a lane.
+__global__ void k_learn_loss(const double* __restrict__ sums, int np, float inv_wsum,
+                             float* __restrict__ idft, float* __restrict__ loss, float* __restrict__ ge) {
     const int lane = threadIdx.x;
-    float e[2], num = 0.f, den = 0.f;
+    double e[2], num = 0.0, den = 0.0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int P = lane + 32 * h;
-        const float d = P < np ? idft[2 * P + 1] : 0.f;
-        e[h] = P < np ? idft[2 * P] - d : 0.f;
+        const double i = P < np ? sums[2 * P] : 0.0, d = P < np ? sums[2 * P + 1] : 0.0;
+        if (P < np) {
+            idft[2 * P] = (float)i;
+            idft[2 * P + 1] = (float)d;
+        }
+        e[h] = i - d;
         num += e[h] * e[h];
         den += d * d;
     }
@@ -324,11 +338,11 @@ __global__ void k_learn_loss(const float* __restrict__ idft, int np, float inv_w
         num += __shfl_xor_sync(0xffffffffu, num, o);
         den += __shfl_xor_sync(0xffffffffu, den, o);
     }
-    den = fmaxf(den, 1e-30f);
-    if (lane == 0) *loss = num / den;
+    den = fmax(den, 1e-30);
+    if (lane == 0) *loss = (float)(num / den);
 #pragma unroll
     for (int h = 0; h < 2; ++h)
-        if (lane + 32 * h < np) ge[lane + 32 * h] = 2.f * e[h] / den * inv_wsum;
+        if (lane + 32 * h < np) ge[lane + 32 * h] = (float)(2.0 * e[h] / den * inv_wsum);
 }
 
 // *p += v, as one reduction of four floats where the caller's table is 16-byte aligned
@@ -424,6 +438,7 @@ struct rick_learn {
     float2* d_wv = nullptr;
     unsigned char* d_field = nullptr;  // a field's constants: sources, probes, plane phasors
     float* d_idft = nullptr;  // [2 * kMaxProbes]
+    double* d_sums = nullptr; // [2 * kMaxProbes], the same before rounding
     float* d_ge = nullptr;
     KbTaps kb4;  // fitted support-4 Kaiser-Bessel taps the correction adds to
 };
@@ -435,6 +450,7 @@ void learn_free(rick_learn* Lr) {
     cudaFree(Lr->d_wv);
     cudaFree(Lr->d_field);
     cudaFree(Lr->d_idft);
+    cudaFree(Lr->d_sums);
     cudaFree(Lr->d_ge);
 }
 
@@ -495,6 +511,7 @@ rick_status rick_learn_create(const rick_config* cfg, int32_t lattice, const dou
     chk(cudaMalloc(&Lr->d_wv, sizeof(float2) * nvis));
     chk(cudaMalloc(&Lr->d_field, field_bytes(Nw)));
     chk(cudaMalloc(&Lr->d_idft, sizeof(float) * 2 * kMaxProbes));
+    chk(cudaMalloc(&Lr->d_sums, sizeof(double) * 2 * kMaxProbes));
     chk(cudaMalloc(&Lr->d_ge, sizeof(float) * kMaxProbes));
     if (e == cudaSuccess) chk(cudaMemset(cnt, 0, sizeof(unsigned) * Nw * 2));
     if (e == cudaSuccess) {
@@ -651,6 +668,7 @@ rick_status rick_learn_field_grad(rick_learn* Lr, const float* table, const floa
     const Probe* d_probes = reinterpret_cast<const Probe*>(d_src + kMaxSources);
     const float2* d_ph = reinterpret_cast<const float2*>(d_probes + kMaxProbes);
     chk(cudaMemsetAsync(Lr->d_idft, 0, sizeof(float) * 2 * kMaxProbes, st));
+    chk(cudaMemsetAsync(Lr->d_sums, 0, sizeof(double) * 2 * kMaxProbes, st));
     LearnConst C{N, Nw, L, Lr->nvis, ns, np, (float)(1.0 / Lr->wsum)};
     if (e == cudaSuccess && Lr->nvis > 0) {
         k_learn_predict<<<(Lr->nvis + 255) / 256, 256, 0, st>>>(Lr->d_vis, C, d_src, Lr->d_wv);
@@ -663,8 +681,8 @@ rick_status rick_learn_field_grad(rick_learn* Lr, const float* table, const floa
         chk(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_learn_forward, 256, fwd));
         if (e == cudaSuccess) {
             const int blocks = std::min((Lr->nvis + kFwdVis - 1) / kFwdVis, sms * std::max(per_sm, 1));
-            k_learn_forward<<<blocks, 256, fwd, st>>>(Lr->d_vis, Lr->d_wv, table, C, Lr->kb4, d_probes, d_ph, Lr->d_idft);
-            k_learn_loss<<<1, 32, 0, st>>>(Lr->d_idft, np, C.inv_wsum * grad_scale, loss, Lr->d_ge);
+            k_learn_forward<<<blocks, 256, fwd, st>>>(Lr->d_vis, Lr->d_wv, table, C, Lr->kb4, d_probes, d_ph, Lr->d_sums);
+            k_learn_loss<<<1, 32, 0, st>>>(Lr->d_sums, np, C.inv_wsum * grad_scale, Lr->d_idft, loss, Lr->d_ge);
         }
         chk(cudaGetLastError());
         if (table_grad) {

@@ -123,9 +123,9 @@ ISSUE_PEAK = 152 * 4 * 2.07e9
 # Shared-memory wavefronts and warp instructions of k_grid per gridded
 # visibility, read from the ncu capture named (KB S = 8, tile 32, fold).
 GRID_COUNTERS = {
-    "large": {"smem_wavefronts": 22352736 / 1109055, "warp_instructions": 129622991 / 1109055,
+    "large": {"smem_wavefronts": 21345410 / 1109055, "warp_instructions": 63448745 / 1109055,
               "profile": "profiles/kernels_meerkat_large_small_16384sq_4w_1ch.md"},
-    "meerkat": {"smem_wavefronts": 39608540 / 1915168, "warp_instructions": 235383545 / 1915168,
+    "meerkat": {"smem_wavefronts": 37985053 / 1915168, "warp_instructions": 119565550 / 1915168,
                 "profile": "profiles/grid_rows_meerkat_small_4096sq_32w_2ch.md"},
 }
 

@@ -136,7 +136,7 @@ __global__ void k_schedule(GridParams G, const uint32_t* __restrict__ offsets,
     for (uint32_t base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < G.n_items;
          base += stride) {
         const uint32_t item = base + lane;
-        int level = 3;
+        int level = 4;   // no list: an empty tile, or beyond the launch's last one
         if (item < G.n_items) {
             uint32_t b[8];
 #pragma unroll

@@ -13,16 +13,24 @@
 // kRun records, so that no warp scans empty tiles and a dense tile is shared.  One
 // warp per entry copies the tile's (T + S - 1)^2 region of the plane (rows and
 // columns taken mod N, which only the fold's footprints ending on cell N use) into
-// its shared buffer with asynchronous copies, all in flight together.  Supports 4 to
-// 8 then predict record by record with the whole warp: lane r evaluates the taps of
-// record r of a batch of 32 into a slot; per record a lane takes the cells (a, rl)
-// and (a, rl + 4) of the footprint, free of bank conflicts, and the 32 partial sums
-// of eight records are added by a transposing butterfly (18 shuffles for eight
-// complex sums).  Other supports predict one record per lane.
+// its shared buffer with asynchronous copies, all in flight together, and predicts
+// the records one per lane: 2S tap polynomials (the tap index is the same in all
+// lanes, so the coefficients are constant-bank operands), then one chain of fused
+// multiply-adds along every footprint row and one over the rows.
 //
-// Measured on GB300 against one record a lane at random bank offsets, every tile
-// visited in turn from an atomic queue: 15.3 M records on 8 x 16 planes of 4096^2
-// 2.01 -> 0.92 ms, 30 k records on 9 planes of 512^2 102 -> 12.5 us (S = 7).
+// The chains are kept for their rounding: on planes amplified by 1/taper the
+// neighbouring terms of a row cancel, and one rounding a cell at the running sum is
+// all that the FP32 result then carries.  Spreading a footprint over the lanes
+// (products rounded one by one, then a butterfly of adds) reads shared memory
+// without bank conflicts, but its sum was 2.1, 1.8, 1.6, 1.4 and 1.3 times as far from
+// 64 bits at supports 8 to 4 on a bare mesh, and it was not faster:
+//
+// Measured on GB300, 15.3 M records on 8 x 16 planes of 4096^2 (S = 8): 0.78 ms
+// here, 0.94 ms spread over the lanes, 2.01 ms one record a lane with every tile
+// visited in turn from an atomic queue and its region copied through registers.  The
+// random row starts of 16 records a half-warp cost about three shared-memory
+// wavefronts a cell where one is the least: 190 M, 0.6 of the 0.78 ms.  The row pitch
+// (T + S - 1 plus 1, 2 or 3) does not matter for them.
 #include <algorithm>
 
 #include "rick_internal.cuh"
@@ -33,7 +41,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRun = 1024;       // records of one entry at most
-constexpr int kTapSlot = 20;     // 80 bytes a record: 16-byte stores of 8 lanes on distinct banks
 
 // g(a + 1 - S/2 - f) for footprint tap a (warp-uniform), by Horner in t = 2 f - 1.
 __device__ __forceinline__ float tap_poly_uniform(const GridParams& G, int a, float t) {
@@ -43,8 +50,18 @@ __device__ __forceinline__ float tap_poly_uniform(const GridParams& G, int a, fl
     return acc;
 }
 
-__host__ __device__ constexpr int region_pitch(int T) { return T + 8; }   // cells; rows rl, rl + 1 are 16 banks apart
-__host__ __device__ constexpr bool by_warp(int SS) { return SS >= 4 && SS <= 8; }
+__host__ __device__ constexpr int region_pitch(int T, int S) { return T + S; }   // cells
+
+// x v + c on both words, one packed instruction (the roundings of two fmaf)
+__device__ __forceinline__ float2 fma_both(float x, float2 v, float2 c) {
+    const float2 xx = make_float2(x, x);
+    uint64_t rd;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(rd)
+        : "l"(*reinterpret_cast<const uint64_t*>(&xx)), "l"(*reinterpret_cast<const uint64_t*>(&v)),
+          "l"(*reinterpret_cast<const uint64_t*>(&c)));
+    return *reinterpret_cast<float2*>(&rd);
+}
 
 // First and last record of tile `item`'s own bins.
 __device__ __forceinline__ uint2 own_records(const GridParams& G, const uint32_t* __restrict__ offsets, uint32_t item) {
@@ -97,11 +114,9 @@ __global__ void k_degrid(GridParams G, const uint32_t* __restrict__ offsets,
     constexpr int kS = SS > 0 ? SS : kMaxSupport;
     const int S = SS > 0 ? SS : G.S;
     const int T = G.T, N = G.N, NT = G.NT;
-    const int R = T + S - 1, RP = by_warp(SS) ? region_pitch(T) : R + 1;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int R = T + S - 1, RP = region_pitch(T, S);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float2* region = reinterpret_cast<float2*>(smem) + (size_t)warp * R * RP;
-    float* slots = smem + (size_t)nw * 2 * ((R * RP + 1) & ~1) + warp * 32 * kTapSlot;
-    if (by_warp(SS)) region = reinterpret_cast<float2*>(smem) + (size_t)warp * ((R * RP + 1) & ~1);
     const uint32_t tiles = (uint32_t)NT * NT, n_entries = min(__ldg(work_counter + 1), G.entry_cap);
     constexpr float kInvFrac = 1.0f / 16777216.0f;
 
@@ -127,103 +142,42 @@ __global__ void k_degrid(GridParams G, const uint32_t* __restrict__ offsets,
                 for (int rr = 0; rr < R; ++rr) copy(rr, x + lane);
         if (S > 1)
             for (int q = lane; q < R * (S - 1); q += 32) copy(q / (S - 1), T + q % (S - 1));
+        const uint32_t re = min(e.y + (uint32_t)kRun, own_records(G, offsets, item).y);
+        VisRecord rec = {};
+        if (e.y + lane < re) rec = records[e.y + lane];
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
-        const uint32_t re = min(e.y + (uint32_t)kRun, own_records(G, offsets, item).y);
-        for (uint32_t base = e.y; base < re; base += 32u) {
-            const uint32_t r = base + lane;
-            VisRecord rec = {};
-            if (r < re) rec = records[r];
-            const int il = (int)(rec.px >> kFracBits), jl = (int)(rec.py >> kFracBits);
-            const float tx2 = fmaf(2.0f, (float)(rec.px & kFracMask) * kInvFrac, -1.0f);
-            const float ty2 = fmaf(2.0f, (float)(rec.py & kFracMask) * kInvFrac, -1.0f);
+        for (uint32_t r = e.y + lane; r < re; r += 32u) {
+            const VisRecord cur = rec;
+            if (r + 32u < re) rec = records[r + 32u];   // the lane's next record, in flight meanwhile
+            const int il = (int)(cur.px >> kFracBits), jl = (int)(cur.py >> kFracBits);
+            const float tx2 = fmaf(2.0f, (float)(cur.px & kFracMask) * kInvFrac, -1.0f);
+            const float ty2 = fmaf(2.0f, (float)(cur.py & kFracMask) * kInvFrac, -1.0f);
             // (-1)^(i0 + j0) of the footprint's first cell (T is even)
             const float s0 = ((il + jl) & 1) ? -1.f : 1.f;
-            if constexpr (by_warp(SS)) {
-                // taps with the checkerboard folded in; zero beyond the support
-                float gx[8], gy[8];
+            // 1-D taps with the checkerboard folded in: (-1)^a, (-1)^b
+            float gx[kS], gy[kS];
 #pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const float sa = (t & 1) ? -1.f : 1.f;
-                    gx[t] = t < SS ? s0 * sa * tap_poly_uniform(G, t, tx2) : 0.f;
-                    gy[t] = t < SS ? sa * tap_poly_uniform(G, t, ty2) : 0.f;
+            for (int a = 0; a < kS; ++a) {
+                if (a < S) {
+                    const float sa = (a & 1) ? -1.f : 1.f;
+                    gx[a] = s0 * sa * tap_poly_uniform(G, a, tx2);
+                    gy[a] = sa * tap_poly_uniform(G, a, ty2);
                 }
-                float* mine = slots + lane * kTapSlot;
-                *reinterpret_cast<float4*>(mine) = make_float4(gx[0], gx[1], gx[2], gx[3]);
-                *reinterpret_cast<float4*>(mine + 4) = make_float4(gx[4], gx[5], gx[6], gx[7]);
-                *reinterpret_cast<float4*>(mine + 8) = make_float4(gy[0], gy[4], gy[1], gy[5]);
-                *reinterpret_cast<float4*>(mine + 12) = make_float4(gy[2], gy[6], gy[3], gy[7]);
-                __syncwarp();
-                // this lane's cells: beyond the support the last one, times zero
-                const int a = lane & 7, rl = lane >> 3;
-                const float2* c0 = region + min(rl, SS - 1) * RP + min(a, SS - 1);
-                const float2* c1 = region + min(rl + 4, SS - 1) * RP + min(a, SS - 1);
-                const int first = jl * RP + il, cnt = (int)min(32u, re - base);
-                for (int q0 = 0; q0 < cnt; q0 += 8) {
-                    float2 v[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {   // slots beyond cnt hold records of zero position and taps
-                        const int at = __shfl_sync(kFull, first, q0 + q);
-                        const float x = slots[(q0 + q) * kTapSlot + a];
-                        const float2 y = *reinterpret_cast<const float2*>(slots + (q0 + q) * kTapSlot + 8 + 2 * rl);
-                        const float2 f0 = c0[at], f1 = c1[at];
-                        v[q].x = x * fmaf(y.y, f1.x, y.x * f0.x);
-                        v[q].y = x * fmaf(y.y, f1.y, y.x * f0.y);
-                    }
-                    // sum over the lanes: after the three halving steps lane bits 4, 3, 2
-                    // name the record, after the last two every lane of it has the sum
-#pragma unroll
-                    for (int h = 4; h >= 1; h >>= 1) {
-                        const bool upper = (lane & (4 * h)) != 0;
-#pragma unroll
-                        for (int q = 0; q < h; ++q) {
-                            const float2 give = upper ? v[q] : v[q + h], keep = upper ? v[q + h] : v[q];
-                            v[q].x = keep.x + __shfl_xor_sync(kFull, give.x, 4 * h);
-                            v[q].y = keep.y + __shfl_xor_sync(kFull, give.y, 4 * h);
-                        }
-                    }
-#pragma unroll
-                    for (int o = 2; o >= 1; o >>= 1) {
-                        v[0].x += __shfl_xor_sync(kFull, v[0].x, o);
-                        v[0].y += __shfl_xor_sync(kFull, v[0].y, o);
-                    }
-                    const int rq = q0 + (lane >> 2);
-                    const uint32_t index = __shfl_sync(kFull, __float_as_uint(rec.wv_re), rq);
-                    const float weight = __shfl_sync(kFull, rec.wv_im, rq);
-                    if ((lane & 3) == 0 && rq < cnt) store_prediction(G, vis_out, index, weight, v[0]);
-                }
-                __syncwarp();   // the slots are rewritten
-            } else if (r < re) {
-                // 1-D taps with the checkerboard folded in: (-1)^a, (-1)^b
-                float gx[kS], gy[kS];
-#pragma unroll
-                for (int a = 0; a < kS; ++a) {
-                    if (a < S) {
-                        const float sa = (a & 1) ? -1.f : 1.f;
-                        gx[a] = s0 * sa * tap_poly_uniform(G, a, tx2);
-                        gy[a] = sa * tap_poly_uniform(G, a, ty2);
-                    }
-                }
-                float2 acc = make_float2(0.f, 0.f);
-                const float2* row = region + jl * RP + il;
-#pragma unroll
-                for (int b = 0; b < kS; ++b) {
-                    if (b < S) {
-                        float2 rs = make_float2(0.f, 0.f);
-#pragma unroll
-                        for (int a = 0; a < kS; ++a) {
-                            if (a < S) {
-                                const float2 f = row[b * RP + a];
-                                rs.x = fmaf(gx[a], f.x, rs.x);
-                                rs.y = fmaf(gx[a], f.y, rs.y);
-                            }
-                        }
-                        acc.x = fmaf(gy[b], rs.x, acc.x);
-                        acc.y = fmaf(gy[b], rs.y, acc.y);
-                    }
-                }
-                store_prediction(G, vis_out, __float_as_uint(rec.wv_re), rec.wv_im, acc);
             }
+            float2 acc = make_float2(0.f, 0.f);
+            const float2* row = region + jl * RP + il;
+#pragma unroll
+            for (int b = 0; b < kS; ++b) {
+                if (b < S) {
+                    float2 rs = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int a = 0; a < kS; ++a)
+                        if (a < S) rs = fma_both(gx[a], row[b * RP + a], rs);
+                    acc = fma_both(gy[b], rs, acc);
+                }
+            }
+            store_prediction(G, vis_out, __float_as_uint(cur.wv_re), cur.wv_im, acc);
         }
         __syncwarp();  // the region is rewritten for the next entry
     }
@@ -233,9 +187,8 @@ template <int SS>
 cudaError_t launch_degrid_one(const GridParams& G, const uint32_t* offsets, const VisRecord* records,
                               const float2* grids, float2* vis_out, uint32_t* counter, int threads,
                               int num_sms, cudaStream_t stream) {
-    const int R = G.T + G.S - 1, RP = by_warp(SS) ? region_pitch(G.T) : R + 1;
-    const size_t smem = (size_t)(threads / 32) * (sizeof(float2) * ((R * RP + 1) & ~1) +
-                                                  (by_warp(SS) ? sizeof(float) * 32 * kTapSlot : 0));
+    const int R = G.T + G.S - 1;
+    const size_t smem = (size_t)(threads / 32) * R * region_pitch(G.T, G.S) * sizeof(float2);
     auto fn = k_degrid<SS>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

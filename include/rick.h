@@ -184,8 +184,9 @@ typedef struct rick_plan rick_plan;
  * cuFFT plans -- or, with the library's own transform (RICK_FFT_OWN), its
  * twiddle tables, the per-pixel table of the fused row passes (the phase of
  * stored plane 0 and the plane step as Q0.32 turns, and the imaging and model
- * scales: 16 bytes per image pixel, computed once in FP64 on the device) and
- * the occupancy masks used for pruning.  The current CUDA device is the
+ * scales: 16 bytes per image pixel, computed once in FP64 on the device; and the
+ * next 32 bits of the turns for one quadrant, which the separate reduction adds:
+ * 2 bytes per image pixel) and the occupancy masks used for pruning.  The current CUDA device is the
  * plan's device.  On failure *out is NULL and nothing is leaked. */
 rick_status rick_plan_create(const rick_config* cfg, rick_plan** out);
 

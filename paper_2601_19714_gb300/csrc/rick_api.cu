@@ -244,6 +244,7 @@ struct rick_plan {
     uint32_t* d_tileocc = nullptr;   // [C][planes][NT][ceil(NT/32)] tile bits
     uint32_t* d_collist = nullptr;   // 2 + [C][planes][NT]: reached tile columns (Occupancy::list)
     uint2* d_pix_turns = nullptr;    // fused row passes: per-pixel turns and scales [N][N]
+    uint2* d_pix_low = nullptr;      // the turns' next 32 bits, one quadrant
     float* d_pix_scale = nullptr;
     float* d_pix_model_scale = nullptr;
     // w-kernel: tap polynomials and the constants of its transform C_w
@@ -270,6 +271,7 @@ void release(rick_plan* P) {
     dfree(P->d_tileocc);
     dfree(P->d_collist);
     dfree(P->d_pix_turns);
+    dfree(P->d_pix_low);
     dfree(P->d_pix_scale);
     dfree(P->d_pix_model_scale);
     dfree(P->d_density);
@@ -549,10 +551,11 @@ rick_status plan_init(rick_plan* P, const rick_config* cfg) {
         P->light_cap = (uint32_t)(P->nkeys / 4);
         RK_CUDA(dmalloc(&P->d_light, sizeof(uint32_t) * (size_t)P->light_cap));
         RK_CUDA(dmalloc(&P->d_pix_turns, sizeof(uint2) * NN));
+        RK_CUDA(dmalloc(&P->d_pix_low, sizeof(uint2) * (size_t)(c.N / 2 + 1) * (c.N / 2 + 1)));
         RK_CUDA(dmalloc(&P->d_pix_scale, sizeof(float) * NN));
         RK_CUDA(dmalloc(&P->d_pix_model_scale, sizeof(float) * NN));
-        RK_CUDA(launch_pixel_phase(phase_params(P, 0, 1, 0, 1), P->d_inv_taper, P->d_pix_turns, P->d_pix_scale,
-                                   P->d_pix_model_scale, nullptr));
+        RK_CUDA(launch_pixel_phase(phase_params(P, 0, 1, 0, 1), P->d_inv_taper, P->d_pix_turns, P->d_pix_low,
+                                   P->d_pix_scale, P->d_pix_model_scale, nullptr));
         RK_CUDA(cudaDeviceSynchronize());
         return RICK_OK;   // no cuFFT plans
     }
@@ -895,7 +898,7 @@ rick_status phase_impl(rick_plan* P, const float* grids, int c0, int c1, int k0,
     int launches = 0;
     rick_status s = check_launch(
         launch_phase_reduce(pp, reinterpret_cast<const float2*>(grids), weight_sum + c0,
-                            P->d_inv_taper, P->d_pix_turns, P->d_pix_scale, image_real,
+                            P->d_inv_taper, P->d_pix_turns, P->d_pix_low, P->d_pix_scale, image_real,
                             reinterpret_cast<float2*>(image_complex), st, &launches),
         "phase kernel");
     P->launches += launches;

@@ -354,6 +354,12 @@ __device__ __forceinline__ uint32_t turns_q32(double t) {
     return (uint32_t)__double2ull_rz(f * 4294967296.0);
 }
 
+// the 32 bits after those (0 where t is a hair below an integer, whose fraction rounds to 1)
+__device__ __forceinline__ uint32_t turns_low(double t) {
+    const double f = (t - floor(t)) * 4294967296.0;
+    return (uint32_t)__double2ull_rz((f - floor(f)) * 4294967296.0);
+}
+
 __device__ __forceinline__ uint32_t turns_q32f(float t) {
     const float f = t - floorf(t);
     return (uint32_t)__float2ull_rz(f * 4294967296.0f);
@@ -365,11 +371,12 @@ __device__ __forceinline__ uint32_t turns_q32f(float t) {
 //     the plane step dw (n - 1) in turns, Q0.32 fixed point (FP64 -- or FP32
 //     under RICK_PREC_ALL_FP32 -- from n - 1 = -(l^2 + m^2)/(1 + n)), so that
 //     plane k's phase is t_0 + k dt, exact modulo one turn;
+//   low[|q - N/2| (N/2 + 1) + |p - N/2|], their next 32 bits (FP64 only),
 //   scale[q N + p] = (-1)^(p+q) n / (C(p) C(q) C_w) (imaging),
 //   model_scale[q N + p] = (-1)^(p+q) / (n C(p) C(q) C_w) (prediction).
 // P describes stored plane 0 (w_first = its w).
 __global__ void k_pixel_phase(PhaseParams P, const float* __restrict__ inv_taper, uint2* __restrict__ turns,
-                              float* __restrict__ scale, float* __restrict__ model_scale) {
+                              uint2* __restrict__ low, float* __restrict__ scale, float* __restrict__ model_scale) {
     const int N = P.Ni, halfN = N / 2;   // image pixels (the central Ni x Ni of a padded mesh)
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)N * N) return;
@@ -385,6 +392,9 @@ __global__ void k_pixel_phase(PhaseParams P, const float* __restrict__ inv_taper
         turns[i] = make_uint2(turns_q32f((float)P.w_first * df), turns_q32f((float)P.dw * df));
     } else {
         turns[i] = make_uint2(turns_q32(P.w_first * delta), turns_q32(P.dw * delta));
+        if (p <= halfN && q <= halfN)
+            low[(size_t)(halfN - q) * (halfN + 1) + (halfN - p)] =
+                make_uint2(turns_low(P.w_first * delta), turns_low(P.dw * delta));
     }
     const float sg = ((p + q) & 1) ? -1.f : 1.f;
     const float c = sg * inv_taper[p] * inv_taper[q] * w_taper_inv(P, delta);
@@ -1398,10 +1408,10 @@ cudaError_t launch_model_rows(const PhaseParams& P, const float* image, const ui
     return e;
 }
 
-cudaError_t launch_pixel_phase(const PhaseParams& P0, const float* inv_taper, uint2* turns, float* scale,
-                               float* model_scale, cudaStream_t st) {
+cudaError_t launch_pixel_phase(const PhaseParams& P0, const float* inv_taper, uint2* turns, uint2* low,
+                               float* scale, float* model_scale, cudaStream_t st) {
     const int64_t n = (int64_t)P0.Ni * P0.Ni;
-    k_pixel_phase<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(P0, inv_taper, turns, scale, model_scale);
+    k_pixel_phase<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(P0, inv_taper, turns, low, scale, model_scale);
     return cudaGetLastError();
 }
 

@@ -248,10 +248,11 @@ cudaError_t launch_grid(const GridParams& G, const uint32_t* offsets, const VisR
                         float2* grids, uint32_t* work_counter, int threads, int num_sms,
                         cudaStream_t stream, int* launches);
 
-// pix_turns, pix_scale: the plan's per-pixel table (launch_pixel_phase), or null
+// pix_turns, pix_low, pix_scale: the plan's per-pixel tables (launch_pixel_phase), or null
 cudaError_t launch_phase_reduce(const PhaseParams& P, const float2* grids, const double* wsum,
-                                const float* taper, const uint2* pix_turns, const float* pix_scale,
-                                float* image_real, float2* image_complex, cudaStream_t stream, int* launches);
+                                const float* taper, const uint2* pix_turns, const uint2* pix_low,
+                                const float* pix_scale, float* image_real, float2* image_complex,
+                                cudaStream_t stream, int* launches);
 
 // prediction (degridding)
 cudaError_t launch_model_planes(const PhaseParams& P, const float* image, const float* inv_taper,
@@ -334,9 +335,11 @@ cudaError_t launch_rows_phase_reduce(const PhaseParams& P, const float2* grids, 
 // The per-pixel table of the fused row passes ([N][N] each): the phase of
 // stored plane 0 and the plane step in Q0.32 turns, and the pixel's scale for
 // imaging (checkerboard sign, n, tapers) and for the model of a prediction
-// (sign, 1/n, tapers); P0 = the phase parameters of stored plane 0.
-cudaError_t launch_pixel_phase(const PhaseParams& P0, const float* inv_taper, uint2* turns, float* scale,
-                               float* model_scale, cudaStream_t stream);
+// (sign, 1/n, tapers); P0 = the phase parameters of stored plane 0.  low[b][a], a, b
+// <= N/2: the next 32 bits of both turns at the pixels (N/2 +- a, N/2 +- b) (not
+// written under RICK_PREC_ALL_FP32).
+cudaError_t launch_pixel_phase(const PhaseParams& P0, const float* inv_taper, uint2* turns, uint2* low,
+                               float* scale, float* model_scale, cudaStream_t stream);
 // Prediction: the model rows of image[nc][N][N] for the launch's planes,
 // transformed along the rows (forward), into grids[nc][nk][N][N]; with occ,
 // unreached planes are skipped and only reached tile columns written.

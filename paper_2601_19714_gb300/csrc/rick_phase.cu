@@ -13,8 +13,9 @@
 // Phase (pattern 1, FP64 only where it is needed): per pixel, in FP64,
 //   delta = n - 1 = -(l^2 + m^2)/(1 + n)          (no cancellation)
 //   t_0 = frac(w_first * delta), dt = frac(dw * delta)   [turns]
-// both converted to 64-bit fixed point (Q0.64), so that t_k = t_0 + k dt is
-// exact modulo one turn with integer adds.  Every 8th plane the phasor is
+// both converted to 64-bit fixed point (Q0.64; with the library's own transform
+// once, at plan creation), so that t_k = t_0 + k dt is exact modulo one turn with
+// integer adds.  Every 8th plane the phasor is
 // formed exactly from the top 32 bits (sincospif of a value in [-1, 1)); in
 // between it advances by one FP32 complex multiply with exp(2 pi i dt).  The
 // only FP64 work is a handful of operations per pixel, never per plane.
@@ -47,16 +48,20 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 
-
-// TABLES: the plan has the per-pixel turns (Q0.32, of stored plane 0 and of the plane
-// step) and scales of the fused row pass; reading those 12 bytes per pixel takes the
-// place of the FP64 set-up, which kept the kernel from HBM speed (16 planes of 4096^2
-// on GB300: 1.17 -> 0.38 ms).
+// TABLES: the plan has the per-pixel turns (of stored plane 0 and of the plane step)
+// and scales; reading them takes the place of the FP64 set-up, which kept the kernel
+// from HBM speed (16 planes of 4096^2 on GB300: 1.18 ms with it, 0.38 ms from the
+// tables).  The upper 32 bits of the turns and the scale are those of the fused row
+// pass (12 bytes a pixel); the lower 32 bits, without which plane k's phase would be
+// up to k 2^-32 turns off, are a quadrant's (they depend on |p - N/2| and |q - N/2|
+// only): 2 bytes a pixel of memory, and mostly cache hits.
+// From the tables, four CTAs an SM (64 registers; left to itself the compiler takes
+// 85, two CTAs, 0.51 ms).
 template <int PREC, bool COMPLEX_OUT, bool TABLES>
-__global__ void __launch_bounds__(kPhaseThreads)
+__global__ void __launch_bounds__(kPhaseThreads, TABLES ? 4 : PREC == RICK_PREC_ALL_FP32 ? 6 : 3)
 k_phase_reduce(PhaseParams P, const float2* __restrict__ grids, const double* __restrict__ wsum,
                const float* __restrict__ inv_taper, const uint2* __restrict__ pix_turns,
-               const float* __restrict__ pix_scale, float* __restrict__ image_real,
+               const uint2* __restrict__ pix_low, const float* __restrict__ pix_scale, float* __restrict__ image_real,
                float2* __restrict__ image_complex) {
     // (p, q): image pixel; the planes are Ng x Ng with the image at offset off
     const int N = P.N, Ni = P.Ni, halfN = Ni / 2;
@@ -73,11 +78,12 @@ k_phase_reduce(PhaseParams P, const float2* __restrict__ grids, const double* __
         const size_t at = (size_t)q * Ni + p;   // p even: the pair is 16- and 8-byte aligned
         const uint4 t = __ldcs(reinterpret_cast<const uint4*>(pix_turns + at));
         const float2 s2 = __ldcs(reinterpret_cast<const float2*>(pix_scale + at));
-        const uint32_t k0 = (uint32_t)P.k_first;
-        t0[0] = (uint64_t)(t.x + k0 * t.y) << 32;
-        t0[1] = (uint64_t)(t.z + k0 * t.w) << 32;
-        dt[0] = (uint64_t)t.y << 32;
-        dt[1] = (uint64_t)t.w << 32;
+        const uint2* low = pix_low + (size_t)abs(q - halfN) * (halfN + 1);
+        const uint2 w0 = __ldg(low + abs(p - halfN)), w1 = __ldg(low + abs(p + 1 - halfN));
+        dt[0] = (uint64_t)t.y << 32 | w0.y;
+        dt[1] = (uint64_t)t.w << 32 | w1.y;
+        t0[0] = ((uint64_t)t.x << 32 | w0.x) + (uint64_t)P.k_first * dt[0];
+        t0[1] = ((uint64_t)t.z << 32 | w1.x) + (uint64_t)P.k_first * dt[1];
         scale[0] = s2.x;
         scale[1] = s2.y;
     }
@@ -258,14 +264,15 @@ cudaError_t launch_model_planes(const PhaseParams& P, const float* image, const 
 }
 
 cudaError_t launch_phase_reduce(const PhaseParams& P, const float2* grids, const double* wsum,
-                                const float* inv_taper, const uint2* pix_turns, const float* pix_scale,
-                                float* image_real, float2* image_complex, cudaStream_t stream, int* launches) {
+                                const float* inv_taper, const uint2* pix_turns, const uint2* pix_low,
+                                const float* pix_scale, float* image_real, float2* image_complex,
+                                cudaStream_t stream, int* launches) {
     const int64_t threads = (int64_t)P.Ni * (P.Ni / 2);   // every image pixel pair
     const int64_t blocks = (threads + kPhaseThreads - 1) / kPhaseThreads;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     auto run = [&](auto kernel) {
-        kernel<<<(unsigned)blocks, kPhaseThreads, 0, stream>>>(P, grids, wsum, inv_taper, pix_turns, pix_scale,
-                                                               image_real, image_complex);
+        kernel<<<(unsigned)blocks, kPhaseThreads, 0, stream>>>(P, grids, wsum, inv_taper, pix_turns, pix_low,
+                                                               pix_scale, image_real, image_complex);
     };
     const bool cplx = image_complex != nullptr;
     if (P.precision == RICK_PREC_ALL_FP32) {

@@ -228,22 +228,25 @@ __device__ __forceinline__ float2 cell_phasor(int i0, int j0, int p, int q, int 
     return make_float2(c, s);
 }
 
+constexpr size_t kSharedMax = 227 * 1024;   // shared memory of a CTA at most
 constexpr int kFwdVis = 128;   // visibilities staged at a time
 constexpr int kFwdRow = 6;     // float4 of a staged visibility: 16 taps, (W V, fx, fy), (w, i0, j0, k)
 
 // I_P and D_P summed over all visibilities (out[2P], out[2P + 1]): eight warps,
 // four pairs of them taking a quarter of the staged visibilities each, lane l of a
 // pair's first and second warp the probes l and 32 + l.
+template <bool STAGED>
 __global__ void __launch_bounds__(256)
 k_learn_forward(const LearnVis* __restrict__ vis, const float2* __restrict__ wv,
                 const float* __restrict__ table, LearnConst C, KbTaps K, const Probe* __restrict__ probes,
                 const float2* __restrict__ ph, double* __restrict__ out) {
-    extern __shared__ __align__(16) float4 s_vis[];   // kFwdVis rows, then the phasors e^(2 pi i w_k delta_P)
+    extern __shared__ __align__(16) float4 s_vis[];   // kFwdVis rows, then (STAGED) the phasors e^(2 pi i w_k delta_P)
     float2* s_ph = reinterpret_cast<float2*>(s_vis + kFwdVis * kFwdRow);
     __shared__ double2 s_acc[4][kMaxProbes];
     const int tid = threadIdx.x, warp = tid >> 5;
     const int P = (warp & 1) * 32 + (tid & 31), quarter = warp >> 1;
-    for (int i = tid; i < C.Nw * kMaxProbes; i += 256) s_ph[i] = ph[i];
+    if (STAGED)
+        for (int i = tid; i < C.Nw * kMaxProbes; i += 256) s_ph[i] = ph[i];
     Probe pr = {};
     if (P < C.np) pr = probes[P];
     const bool idle = (warp & 1) * 32 >= C.np;
@@ -291,7 +294,8 @@ k_learn_forward(const LearnVis* __restrict__ vis, const float2* __restrict__ wv,
                 S.x = fmaf(g[q].x, pr.sy[q - 1].x, fmaf(-g[q].y, pr.sy[q - 1].y, S.x));
                 S.y = fmaf(g[q].x, pr.sy[q - 1].y, fmaf(g[q].y, pr.sy[q - 1].x, S.y));
             }
-            const float2 u = cmulf(c, s_ph[__float_as_int(b.w) * kMaxProbes + P]);
+            const int at = __float_as_int(b.w) * kMaxProbes + P;
+            const float2 u = cmulf(c, STAGED ? s_ph[at] : __ldg(ph + at));
             img = fmaf(u.x, S.x, fmaf(-u.y, S.y, img));
             // the direct inversion: the rest of its turn, below one
             const float2 d = turn_phasor(fmaf(a.z, pr.pn, fmaf(a.w, pr.qn, fmaf(b.x, pr.delta, pr.turn))));
@@ -362,21 +366,24 @@ __device__ __forceinline__ void add4(float* p, float4 v, bool aligned16) {
 // e^(2 pi i w_k delta_P) E_x(i0 + a) E_y(j0 + b)), spread bilinearly onto the lattice
 // of its plane by vector reductions in L2 (16 of four floats a visibility; FP32
 // shared-memory atomics are compare-and-swap loops).
+template <bool STAGED>
 __global__ void __launch_bounds__(256)
 k_learn_backward(const LearnVis* __restrict__ vis, const float2* __restrict__ wv, LearnConst C,
                  const Probe* __restrict__ probes, const float2* __restrict__ ph, const float* __restrict__ ge,
                  float* __restrict__ table_grad, bool aligned16) {
     __shared__ __align__(16) float4 s_step[kMaxProbes][3];   // sx[0..2], sy[0..2]
     __shared__ int2 s_pq[kMaxProbes];
-    extern __shared__ float2 s_gph[];             // ge_P scale_P e^(2 pi i w_k delta_P)
+    extern __shared__ float2 s_gph[];             // STAGED: ge_P scale_P e^(2 pi i w_k delta_P)
+    __shared__ float s_g[kMaxProbes];             // otherwise: ge_P scale_P
     for (int i = threadIdx.x; i < C.np; i += blockDim.x) {
         const Probe o = probes[i];
         s_step[i][0] = make_float4(o.sx[0].x, o.sx[0].y, o.sx[1].x, o.sx[1].y);
         s_step[i][1] = make_float4(o.sx[2].x, o.sx[2].y, o.sy[0].x, o.sy[0].y);
         s_step[i][2] = make_float4(o.sy[1].x, o.sy[1].y, o.sy[2].x, o.sy[2].y);
         s_pq[i] = make_int2(o.p, o.q);
+        if (!STAGED) s_g[i] = ge[i] * o.scale_img;
     }
-    for (int i = threadIdx.x; i < C.Nw * kMaxProbes; i += blockDim.x) {
+    for (int i = threadIdx.x; STAGED && i < C.Nw * kMaxProbes; i += blockDim.x) {
         const int P = i % kMaxProbes;
         const float g = P < C.np ? ge[P] * probes[P].scale_img : 0.f;
         s_gph[i] = make_float2(g * ph[i].x, g * ph[i].y);
@@ -387,7 +394,7 @@ k_learn_backward(const LearnVis* __restrict__ vis, const float2* __restrict__ wv
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < C.nvis; j += gridDim.x * blockDim.x) {
         const LearnVis v = vis[j];
         const float2 w2 = wv[j];
-        const float2* gph = s_gph + v.k * kMaxProbes;
+        const float2* gph = STAGED ? s_gph + v.k * kMaxProbes : ph + (size_t)v.k * kMaxProbes;
         float gt[16];
 #pragma unroll
         for (int q = 0; q < 16; ++q) gt[q] = 0.f;
@@ -396,7 +403,9 @@ k_learn_backward(const LearnVis* __restrict__ vis, const float2* __restrict__ wv
             const int2 pq = s_pq[P];
             const float4 s0 = s_step[P][0], s1 = s_step[P][1], s2 = s_step[P][2];
             const float2 e = cell_phasor(v.i0, v.j0, pq.x, pq.y, C.N, inv_half_n);
-            const float2 c = cmulf(cmulf(w2, gph[P]), e);
+            float2 f = gph[P];
+            if (!STAGED) f = make_float2(s_g[P] * f.x, s_g[P] * f.y);
+            const float2 c = cmulf(cmulf(w2, f), e);
             const float2 cb[4] = {c, cmulf(c, make_float2(s1.z, s1.w)), cmulf(c, make_float2(s2.x, s2.y)),
                                   cmulf(c, make_float2(s2.z, s2.w))};
 #pragma unroll
@@ -676,24 +685,31 @@ rick_status rick_learn_field_grad(rick_learn* Lr, const float* table, const floa
         chk(cudaGetDevice(&dev));
         chk(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         const size_t ph_bytes = sizeof(float2) * Nw * kMaxProbes;
-        const size_t fwd = ph_bytes + sizeof(float4) * kFwdVis * kFwdRow;
-        chk(cudaFuncSetAttribute(k_learn_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd));
-        chk(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_learn_forward, 256, fwd));
+        // the plane phasors (512 bytes a plane) stay in shared memory while they fit beside
+        // the rest (422 planes); beyond, they are read through the caches
+        const size_t rows = sizeof(float4) * kFwdVis * kFwdRow, fixed = sizeof(double2) * 4 * kMaxProbes;
+        const bool staged = ph_bytes + rows + fixed <= kSharedMax;
+        const size_t fwd = rows + (staged ? ph_bytes : 0);
+        auto forward = staged ? k_learn_forward<true> : k_learn_forward<false>;
+        chk(cudaFuncSetAttribute(forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd));
+        chk(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, forward, 256, fwd));
         if (e == cudaSuccess) {
             const int blocks = std::min((Lr->nvis + kFwdVis - 1) / kFwdVis, sms * std::max(per_sm, 1));
-            k_learn_forward<<<blocks, 256, fwd, st>>>(Lr->d_vis, Lr->d_wv, table, C, Lr->kb4, d_probes, d_ph, Lr->d_sums);
+            forward<<<blocks, 256, fwd, st>>>(Lr->d_vis, Lr->d_wv, table, C, Lr->kb4, d_probes, d_ph, Lr->d_sums);
             k_learn_loss<<<1, 32, 0, st>>>(Lr->d_sums, np, C.inv_wsum * grad_scale, Lr->d_idft, loss, Lr->d_ge);
         }
         chk(cudaGetLastError());
         if (table_grad) {
             const size_t ntg = (size_t)(L + 1) * (L + 1) * 16;
             if (!accumulate) chk(cudaMemsetAsync(table_grad, 0, sizeof(float) * ntg * Nw, st));
-            chk(cudaFuncSetAttribute(k_learn_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ph_bytes));
-            chk(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_learn_backward, 256, ph_bytes));
+            const size_t bwd = staged ? ph_bytes : 0;   // the forward pass's other needs are the larger
+            auto backward = staged ? k_learn_backward<true> : k_learn_backward<false>;
+            chk(cudaFuncSetAttribute(backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd));
+            chk(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, backward, 256, bwd));
             if (e == cudaSuccess) {
                 const int blocks = std::min((Lr->nvis + 255) / 256, sms * std::max(per_sm, 1));
-                k_learn_backward<<<blocks, 256, ph_bytes, st>>>(Lr->d_vis, Lr->d_wv, C, d_probes, d_ph, Lr->d_ge, table_grad,
-                                                                ((uintptr_t)table_grad & 15u) == 0);
+                backward<<<blocks, 256, bwd, st>>>(Lr->d_vis, Lr->d_wv, C, d_probes, d_ph, Lr->d_ge, table_grad,
+                                                   ((uintptr_t)table_grad & 15u) == 0);
             }
             chk(cudaGetLastError());
         }

@@ -202,8 +202,6 @@ struct rick_plan {
     uint32_t* d_counter = nullptr;   // gridder queues and list lengths (8 words)
     uint32_t* d_lists = nullptr;     // longest-first tile lists, 3 x list_cap
     uint32_t list_cap = 0;
-    unsigned char* d_huge = nullptr; // split tiles: entries, counters, partial tiles (GridParams::huge)
-    uint32_t huge_cap = 0;
     uint32_t* d_light = nullptr;     // sparse gridding: the other reached tiles (one per tile of the plan)
     uint32_t light_cap = 0;
     unsigned long long* d_counts = nullptr;
@@ -287,7 +285,6 @@ void release(rick_plan* P) {
     dfree(P->d_partials);
     dfree(P->d_counter);
     dfree(P->d_lists);
-    dfree(P->d_huge);
     dfree(P->d_light);
     dfree(P->d_counts);
     dfree(P->d_status);
@@ -409,10 +406,8 @@ rick_status ensure_vis_capacity(rick_plan* P, int64_t nvis) {
     dfree(P->d_stage);
     dfree(P->d_records);
     dfree(P->d_lists);
-    dfree(P->d_huge);
     P->cap_vis = 0;
     P->list_cap = 0;
-    P->huge_cap = 0;
     const size_t n = (size_t)nvis;
     RK_CUDA(dmalloc(&P->d_key, n * sizeof(uint32_t)));
     RK_CUDA(dmalloc(&P->d_rank, n * sizeof(uint32_t)));
@@ -420,10 +415,7 @@ rick_status ensure_vis_capacity(rick_plan* P, int64_t nvis) {
     RK_CUDA(dmalloc(&P->d_records, n * sizeof(VisRecord)));
     const uint32_t cap = schedule_list_cap(nvis, P->T);
     RK_CUDA(dmalloc(&P->d_lists, 3 * (size_t)cap * sizeof(uint32_t)));
-    const uint32_t hcap = huge_list_cap(nvis, P->T);
-    RK_CUDA(dmalloc(&P->d_huge, huge_bytes(hcap, P->T)));
     P->list_cap = cap;
-    P->huge_cap = hcap;
     P->cap_vis = nvis;
     return RICK_OK;
 }
@@ -780,11 +772,13 @@ rick_status grid_impl(rick_plan* P, int c0, int c1, int k0, int k1, float* grids
     G.grab = (uint32_t)P->grab;
     G.lists = P->d_lists;
     G.list_cap = P->list_cap;
-    if (P->d_huge) {
-        G.huge = reinterpret_cast<uint4*>(P->d_huge);
-        G.huge_part = reinterpret_cast<float4*>(G.huge + P->huge_cap);
-        G.huge_done = reinterpret_cast<uint32_t*>(G.huge_part + (size_t)P->huge_cap * (P->T * P->T / 2));
-        G.huge_cap = P->huge_cap;
+    // the split tiles' entries, partial tiles and counters take the place of the
+    // binning's unsorted records (free once binned), which they always fit
+    G.huge_cap = P->d_stage ? huge_capacity(P->cap_vis, P->T) : 0;
+    if (G.huge_cap > 0) {
+        G.huge = reinterpret_cast<uint4*>(P->d_stage);
+        G.huge_part = reinterpret_cast<float4*>(G.huge + G.huge_cap);
+        G.huge_done = reinterpret_cast<uint32_t*>(G.huge_part + (size_t)G.huge_cap * (P->T * P->T / 2));
     }
     G.w_support = 0;
     G.skip_empty = sparse ? 1 : 0;

@@ -110,8 +110,9 @@ struct GridParams {
     uint32_t list_cap;
     // Optional, with lists: tiles of at least 2 huge_chunk(T) records, split over several
     // CTAs.  work_counter[6] entries (tile, chunk, chunks, the tile's first entry),
-    // huge_cap at most (more: no tile is split), each with a T x T partial tile in
-    // huge_part and, at a tile's first entry, its finished chunks in huge_done.
+    // huge_cap at most (more, which huge_capacity excludes: no tile is split), each
+    // with a T x T partial tile in huge_part and, at a tile's first entry, its finished
+    // chunks in huge_done.
     uint4* huge;
     uint32_t* huge_done;
     float4* huge_part;
@@ -163,9 +164,13 @@ inline uint32_t schedule_list_cap(int64_t max_vis, int T) {
 // its partial tile costs as much to write and read back as a few hundred records.
 __host__ __device__ constexpr uint32_t huge_chunk(int T) { return T > 32 ? 16384u : 4096u; }
 constexpr uint32_t kHugeChunks = 128;   // chunks a tile at most (the last CTA adds them up)
-inline uint32_t huge_list_cap(int64_t max_vis, int T) { return (uint32_t)(2 * max_vis / huge_chunk(T) + 64); }
-// bytes of the split tiles' memory: entries, counters, partial tiles
-inline size_t huge_bytes(uint32_t cap, int T) { return (size_t)cap * (sizeof(uint4) + 16 + sizeof(float2) * T * T); }
+// Entries (with their partial tiles and counters) that the memory of n unsorted
+// records holds.  Needed are at most 6 n / huge_chunk(T) -- a record reaches up to four
+// tiles, and R >= 2 chunks of records round up to at most 1.5 R / chunk entries -- of
+// 8 T^2 + 20 bytes each: 12 n bytes at T = 32 and 64, 3 n at T = 16, of the 16 n.
+inline uint32_t huge_capacity(int64_t n, int T) {
+    return (uint32_t)((uint64_t)n * sizeof(VisRecord) / (sizeof(uint4) + sizeof(float2) * T * T + sizeof(uint32_t)));
+}
 
 // Fit the tap polynomials of a Gaussian or Kaiser-Bessel kernel of support S
 // (param = sigma or beta) into G.coef; returns the largest deviation from the

@@ -22,15 +22,16 @@
 // neighbouring terms of a row cancel, and one rounding a cell at the running sum is
 // all that the FP32 result then carries.  Spreading a footprint over the lanes
 // (products rounded one by one, then a butterfly of adds) reads shared memory
-// without bank conflicts, but its sum was 2.1, 1.8, 1.6, 1.4 and 1.3 times as far from
-// 64 bits at supports 8 to 4 on a bare mesh, and it was not faster:
+// without bank conflicts, but its sum is 2.1, 1.8, 1.6, 1.4 and 1.3 times as far from
+// 64 bits at supports 8 to 4 (both orders restated in FP32, bare mesh of 1024^2; 1.2 to
+// 1.4 times on the GPU at 256^2), and it was not faster:
 //
 // Measured on GB300, 15.3 M records on 8 x 16 planes of 4096^2 (S = 8): 0.78 ms
 // here, 0.94 ms spread over the lanes, 2.01 ms one record a lane with every tile
 // visited in turn from an atomic queue and its region copied through registers.  The
-// random row starts of 16 records a half-warp cost about three shared-memory
-// wavefronts a cell where one is the least: 190 M, 0.6 of the 0.78 ms.  The row pitch
-// (T + S - 1 plus 1, 2 or 3) does not matter for them.
+// random row starts of the 32 records cost bank conflicts: at 958 k records, 27 a
+// reached tile, 17.6 shared-memory wavefronts a record (7.4 of them conflicts) and 38
+// warp instructions.  The row pitch (T + S - 1 plus 1, 2 or 3) does not matter.
 #include <algorithm>
 
 #include "rick_internal.cuh"

@@ -270,14 +270,19 @@ k_fft_rows(float2* __restrict__ grids, const float2* __restrict__ twid) {
 // inputs b + T t2 to outputs b + T j.  first() runs stage 0 and stores; after a
 // barrier rest() runs the others; after free() the buffer may be rewritten.
 //
-// The radix-16 transform above, except N = 256 (radix 4) and the model pass of N = 512
-// (radix 8): 64 threads a row, each value's chain a quarter or half as long, for a row
-// of a small mesh is latency only (16 threads of 16 values took 2.6 us a plane: rows of
-// 8 planes of 256^2 21.5 -> 13.6 us, model rows of 9 planes of 512^2 28.7 -> 22.5 us) --
-// exchanging through two buffers in turn, one barrier an exchange, with all N twiddles
-// W_N^k in the table.  Dense rows (k_fft_rows) are bound by HBM and stay at radix 16
-// (64-thread rows: 128 planes of 512^2 98 -> 110 us at best), and so does the imaging
-// pass of N = 512, which equals the separate calls to the last rounding.
+// The rule: at least 64 threads a row.  From N = 1024 the radix-16 transform above has
+// them; N = 512 takes radix 8 and N = 256 radix 4, so that each value's chain is half or
+// a quarter as long, for a row of a small mesh is latency only (16 threads of 16 values
+// took 2.6 us a plane: rows of 8 planes of 256^2 21.5 -> 13.6 us, model rows of 9 planes
+// of 512^2 28.7 -> 22.5 us).  These exchange through two buffers in turn, one barrier an
+// exchange, with all N twiddles W_N^k in the table.  Two exceptions:
+//   - Dense rows (k_fft_rows) are bound by HBM and stay at radix 16 (64-thread rows:
+//     128 planes of 512^2 98 -> 110 us at best).
+//   - The imaging pass of N = 512 stays at radix 16, although radix 8 measures 23.5 ->
+//     19.6 us (8 planes; 57.9 -> 49.1 us for 32, 19.6 -> 17.4 us with the crop): with
+//     the same transform it agrees with the separate calls to the last rounding, which
+//     the division by the taper magnifies at the edges of a bare mesh.  At N = 256 the
+//     two routes differ in rounding there.
 template <int LOG2N, bool INV>
 struct RowDft {
     using Sh = Shape<LOG2N>;
@@ -370,7 +375,8 @@ __device__ __forceinline__ uint32_t turns_q32f(float t) {
 //   turns[q N + p] = (t_0, dt), the phase w_0 (n - 1) of stored plane 0 and
 //     the plane step dw (n - 1) in turns, Q0.32 fixed point (FP64 -- or FP32
 //     under RICK_PREC_ALL_FP32 -- from n - 1 = -(l^2 + m^2)/(1 + n)), so that
-//     plane k's phase is t_0 + k dt, exact modulo one turn;
+//     plane k's phase modulo one turn is t_0 + k dt, at most (k + 1) 2^-32 turns
+//     short of it (the row passes use these bits only);
 //   low[|q - N/2| (N/2 + 1) + |p - N/2|], their next 32 bits (FP64 only),
 //   scale[q N + p] = (-1)^(p+q) n / (C(p) C(q) C_w) (imaging),
 //   model_scale[q N + p] = (-1)^(p+q) / (n C(p) C(q) C_w) (prediction).
@@ -407,7 +413,8 @@ __global__ void k_pixel_phase(PhaseParams P, const float* __restrict__ inv_taper
 //   image[c][q][p] += (-1)^(p+q) n C_w^-1 / (sum W_c C(p) C(q))
 //                     * Re sum_k F_k[q][p] exp(+2 pi i w_k (n - 1)),
 // where F_k[q][.] is the row DFT of the column-transformed plane k.  Thread b
-// owns pixels p = b + (N/16) j.  With t_k = t_0 + k dt the phase of plane k
+// owns the mesh pixels b + T j (RowDft's T and V; Crop keeps the image's).  With
+// t_k = t_0 + k dt the phase of plane k
 // (turns), the sum over a block of planes k = k0..k1 is
 //   e^(2 pi i t_k1) sum_k F_k z^(k1-k),  z = e^(-2 pi i dt),
 // taken by Horner's rule: acc <- acc z + F_k, one complex multiply-add per
@@ -422,7 +429,6 @@ __global__ void k_pixel_phase(PhaseParams P, const float* __restrict__ inv_taper
 // (acc z + 0), so pruning does not change the arithmetic.
 // The per-pixel turns and scale come from the plan's table (k_pixel_phase).
 // The next row is loaded into registers while the current one is transformed.
-// Two CTAs per SM for N <= 4096 (at most 128 registers).
 // CTAs an SM that the fused row passes are compiled for: 16 warps, i.e. at most
 // 128 registers a thread (with the two CTAs of N = 4096 asked for at every
 // length, N = 2048 took 172 registers and ran 8 warps an SM: with the crop 264 ->
@@ -911,7 +917,7 @@ k_model_rows(PhaseParams P, const float* __restrict__ image, const uint2* __rest
     const bool warp_mask = occ.tshift >= 5 && T >= 32;
     const int lane = b & 31;
     // the tile columns of plane r that the column pass reads: the mask bytes, loaded
-    // before the transform, and the 16 bits, needed after it
+    // before the transform, and the V bits, needed after it
     auto load_mask = [&](int r) -> uint32_t {
         if (occ.col == nullptr) return 0xffffu;
         const uint8_t* cm = occ.col + (size_t)r * occ.NT;

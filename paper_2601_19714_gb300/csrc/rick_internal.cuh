@@ -300,8 +300,9 @@ struct Occupancy {
     int tshift = 0, NT = 1, words = 1;
     // the reached tile columns of the launch as a list: list[0] entries
     // col index p * NT + tx in list[2 ..], list[1] the column pass's work
-    // counter (zeroed with the list); nullptr: the column pass launches one
-    // CTA per column and skips the unreached ones
+    // counter (zeroed with the list).  The column pass prunes by the list alone:
+    // with nullptr it transforms, reads and writes every column of every plane,
+    // so the planes must be whole
     uint32_t* list = nullptr;
     // column pass: false -- the input's unreached tiles are zero (imaging);
     // true -- the input is dense and only the reached tiles of the output are

@@ -22,8 +22,9 @@
 // The work is (visibility, probe) pairs, 64 probes a visibility, bound by
 // instruction issue.  Per pair the forward pass needs one phasor of the footprint's
 // first cell, e^(2 pi i (i0 p + j0 q)/N) -- shared by the image term and the direct
-// inversion, whose phases differ from it by a constant of the probe and a fraction
-// of a turn -- and the taps' two polynomials in the probe's unit steps (-1) e^(2 pi
+// inversion, whose phases differ from it by a constant of the probe, the terms of the
+// cell fractions (below half a turn each) and w (n - 1), formed in FP32: an error of
+// 1e-7 |w (n - 1)| turns -- and the taps' two polynomials in the probe's unit steps (-1) e^(2 pi
 // i p/N), whose powers are the probe's constants (rounded from FP64 on the host).
 // A thread of the forward pass owns one probe and walks visibilities staged in
 // shared memory, so its sums stay in registers; a thread of the backward pass owns
@@ -297,7 +298,7 @@ k_learn_forward(const LearnVis* __restrict__ vis, const float2* __restrict__ wv,
             const int at = __float_as_int(b.w) * kMaxProbes + P;
             const float2 u = cmulf(c, STAGED ? s_ph[at] : __ldg(ph + at));
             img = fmaf(u.x, S.x, fmaf(-u.y, S.y, img));
-            // the direct inversion: the rest of its turn, below one
+            // the direct inversion: the rest of its turn, |w (n - 1)| + 1.5 at most
             const float2 d = turn_phasor(fmaf(a.z, pr.pn, fmaf(a.w, pr.qn, fmaf(b.x, pr.delta, pr.turn))));
             dft = fmaf(c.x, d.x, fmaf(-c.y, d.y, dft));
         }

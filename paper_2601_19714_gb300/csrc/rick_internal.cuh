@@ -160,8 +160,10 @@ inline uint32_t schedule_list_cap(int64_t max_vis, int T) {
 }
 
 // Records of one CTA's share of a split tile at least (half the threshold): four
-// warps add 4096 in about 30 us, so one dense tile no longer outlasts the launch, and
-// its partial tile costs as much to write and read back as a few hundred records.
+// warps add 4096 in about 30 us, so one dense tile is no longer one serial chain, and
+// its partial tile costs as much to write and read back as a few hundred records.  (The
+// gridder's block count follows the tiles alone: on a 256^2 plane, 64 tiles, 32 CTAs
+// take the chunks in turn.)
 __host__ __device__ constexpr uint32_t huge_chunk(int T) { return T > 32 ? 16384u : 4096u; }
 constexpr uint32_t kHugeChunks = 128;   // chunks a tile at most (the last CTA adds them up)
 // Entries (with their partial tiles and counters) that the memory of n unsorted
